@@ -114,6 +114,70 @@ def test_actuator_bit_exact(dtype, low, rec, cuda_device):
         N.gnmr_actuator_destroy(h)
 
 
+# Row lengths (in 16-byte vectors) at the edges of every thread group that can
+# hold a row (4 to 256 threads of 8 vectors), and past the widest.
+GROUP_EDGES = [1, 31, 32, 33, 64, 65, 127, 129, 256, 257, 511, 513, 1023, 1025, 2047, 2048, 2049]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("many", [False, True])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_row_groups_bit_exact(dtype, many, shift, cuda_device):
+    """One unit per row length around each group's edge, in tiles that are
+    full, one row short and one row long; `many` adds so many rows of 513
+    vectors that rows wider than two warps are read twice; `shift` moves the
+    output against the input by that many elements (1, 3: rows element by
+    element).  Every row is compared, of the many ones a random 64."""
+    import torch
+    rng = np.random.default_rng(shift)
+    per = 8 if dtype == "bf16" else 4
+    rows, cols = [], []
+    for v in GROUP_EDGES:
+        group = max(4, 1 << (-(-v // 8) - 1).bit_length())
+        tile = max(1, 256 // group)
+        for k, n in enumerate((v * per, v * per + per - 1, v * per + 1)):
+            rows.append(min(9, tile) + k - 1)
+            cols.append(n)
+    if many:
+        rows.append(8 * 2 * 8 * torch.cuda.get_device_properties(0).multi_processor_count)
+        cols.append(513 * per + 1)
+    rows, cols = np.array(rows, np.int64), np.array(cols, np.int64)
+    off = np.concatenate([[0], np.cumsum(rows * cols + rng.integers(0, 5, len(rows)))[:-1]]).astype(np.int64)
+    total = int(off[-1] + rows[-1] * cols[-1]) + 8
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(cuda_device).manual_seed(7 + shift)
+    d_in = torch.empty(total, dtype=tdt, device=cuda_device).normal_(0.0, 1.0, generator=g)
+    for b in range(0, len(rows), 4):                       # kept rows among the others
+        if rows[b] > 1:
+            d_in[off[b]:off[b] + cols[b]] = 0
+            d_in[off[b] + cols[b] + cols[b] // 2] = float("nan")
+    whole = torch.full((total + 16,), 7.0, dtype=tdt, device=cuda_device)
+    d_out = whole[shift:shift + total]
+    mask = (np.arange(len(rows)) % 3 == 0).astype(np.uint8)
+    d_mask = torch.from_numpy(mask).to(cuda_device)
+    h = N.gnmr_actuator_create(off, rows, cols, N.GNMR_DTYPE_BF16 if dtype == "bf16" else N.GNMR_DTYPE_F32, 0)
+    try:
+        N.gnmr_actuator_apply(h, d_in.data_ptr(), d_out.data_ptr(), total, d_mask.data_ptr(), N.GNMR_FQ_E2M1,
+                              N.GNMR_FQ_E5M2)
+        torch.cuda.synchronize()
+    finally:
+        N.gnmr_actuator_destroy(h)
+    covered = torch.zeros(total, dtype=torch.bool, device=cuda_device)
+    for b in range(len(rows)):
+        at, n = int(off[b]), int(cols[b])
+        covered[at:at + int(rows[b]) * n] = True
+        pick = np.arange(rows[b]) if rows[b] <= 64 else np.sort(rng.choice(rows[b], 64, replace=False))
+        if not len(pick):
+            continue
+        idx = torch.from_numpy((at + pick[:, None] * n + np.arange(n)[None]).reshape(-1)).to(cuda_device)
+        x = _host_bits(d_in[idx]).reshape(len(pick), n)
+        want = oracle.fake_quant(x, N.GNMR_FQ_E5M2 if mask[b] else N.GNMR_FQ_E2M1)
+        got = _host_bits(d_out[idx]).reshape(len(pick), n)
+        bits = np.uint16 if dtype == "bf16" else np.uint32
+        assert np.array_equal(got.view(bits), want.view(bits)), (b, n, int(rows[b]))
+    assert bool((d_out[~covered] == 7.0).all()) and bool((whole[total + shift:] == 7.0).all())
+
+
 def test_actuator_driven_by_gnmr_step(cuda_device):
     """The mask gnmr_step writes selects each unit's activation format."""
     import torch
