@@ -399,6 +399,8 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         const int32_t step_warps = static_cast<int32_t>(std::min<int64_t>(plan.num_runs, grid_warps));
         p.num_warps = step_warps;
         p.num_runs = plan.num_runs;
+        p.pool = variant == gnmr::kVariantSmall && U >= gnmr::kPoolUnitsPerSm * sms &&
+                 U <= gnmr::kPoolUnitsPerWarp * p.num_warps;
         p.window = c.window;
         p.max_o = c.max_o;
         p.lock_len = c.lock_len;

@@ -38,6 +38,14 @@ constexpr int64_t kRunsPerWarp = 16;
 constexpr int64_t kBulkRunMin = int64_t(64) << 10;
 constexpr int64_t kBulkRunMax = int64_t(256) << 10;
 
+// Layouts in which a CTA's warps pool the units of their last epilogue batches:
+// from kPoolUnitsPerSm units per SM to kPoolUnitsPerWarp per warp.  An epilogue
+// batch takes about 0.9 us of an SM's fp64 pipe and 4.4 us of latency, so below
+// about five batches per SM there is nothing to save, and with 20 units a warp
+// (100K units) the batches are full enough: 262.8 us without, 264.4 with.
+constexpr int64_t kPoolUnitsPerSm = 6;
+constexpr int64_t kPoolUnitsPerWarp = 16;
+
 // Persistent per-unit controller state (Algorithm 1 and 2), 40 bytes.
 struct UnitState {
     double mean;      // A_b, historical mean of n_b
@@ -142,6 +150,7 @@ struct StepParams {
     int32_t window;
     int32_t max_o;
     int32_t lock_len;
+    int32_t pool;                // 1: the CTA's warps pool their last units (many units per SM)
     int32_t num_runs;            // R; runs num_warps .. R - 1 are taken dynamically
     int64_t warmup_steps;
     double alpha_init, alpha_main, beta_init, beta_main, eps;

@@ -62,11 +62,13 @@ template <> struct Shape<kVariantSmall> {
     static constexpr int kUnroll = 8;
     static constexpr int kMinCtas = 2;
     static constexpr bool kDynamic = false;           // one planned run per warp
+    static constexpr bool kPool = true;               // may pool the warps' last units
 };
 template <> struct Shape<kVariantBulk> {
     static constexpr int kUnroll = 16;
     static constexpr int kMinCtas = 1;
     static constexpr bool kDynamic = true;            // further runs taken from a counter
+    static constexpr bool kPool = false;
 };
 
 __device__ __forceinline__ double pick_threshold(double override_value, int64_t t, int64_t warmup,
@@ -892,6 +894,83 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
     }
 }
 
+// Where a CTA's warps leave the completed units that did not fill a batch of
+// their own (fewer than 32 each): together they make full batches again.  The
+// fp64 pipe takes a warp instruction every 20 cycles however many of its lanes
+// are active, so the epilogue costs by the batch, and a partly filled one per
+// warp made it most of the step on layouts of a few units per warp (30,000
+// units of 48-4,096 bf16 elements, 6 a warp, fp64 pipe 58 % busy: 42.7 -> 34.4
+// us).  Layouts of fewer units per SM or more per warp don't use the pool
+// (kPoolUnitsPerSm, kPoolUnitsPerWarp): each warp runs its own batch.
+struct EpiloguePool {
+    double sumsq[kThreads];
+    int32_t unit[kThreads];
+    uint32_t count;                  // units left so far
+    uint32_t warps;                  // warps that have left theirs
+    uint32_t num_rest;               // full batches left for after the barrier,
+    uint32_t rest[kWarpsPerCta];     // and which
+    uint32_t fill[kWarpsPerCta];     // units written to batch i (slots 32 i ...)
+};
+constexpr uint32_t kNoBatch = ~0u;
+
+// Leaves the lanes' `n` < 32 units.  If they complete a batch the warp takes it
+// (the lanes' b, s become that batch's, n = 32), else n = 0.  What it does not
+// take (a second batch, and any that the CTA's last warp completes) goes to
+// pool_rest(), with the batch that stays partly filled: one warp each, where
+// the last warp would run them one after the other.  No warp waits.
+__device__ __forceinline__ void pool_leave(EpiloguePool &pool, int here, int &n, int32_t &b, double &s, int lane)
+{
+    uint32_t base = 0;
+    if (lane == 0 && n > 0)
+        base = atomicAdd(&pool.count, static_cast<uint32_t>(n));
+    base = __shfl_sync(kFull, base, 0);
+    if (lane < n) {
+        pool.unit[base + lane] = b;
+        pool.sumsq[base + lane] = s;
+    }
+    __threadfence_block();
+    __syncwarp();
+    uint32_t full = kNoBatch;
+    if (lane == 0) {
+        const uint32_t m = static_cast<uint32_t>(n), first = base / 32, room = 32 - base % 32;
+        const uint32_t m0 = m < room ? m : room;                       // units that went to batch `first`
+        uint32_t full2 = kNoBatch;                                     // later units may be there before earlier ones
+        if (m0 > 0 && atomicAdd(&pool.fill[first], m0) + m0 == 32)
+            full = first;
+        if (m > m0 && atomicAdd(&pool.fill[first + 1], m - m0) + m - m0 == 32)
+            full2 = first + 1;
+        __threadfence_block();
+        const bool last = atomicAdd(&pool.warps, 1u) + 1 == static_cast<uint32_t>(here);
+        if (full2 != kNoBatch)
+            pool.rest[atomicAdd(&pool.num_rest, 1u)] = full2;
+        if (last && full != kNoBatch) {
+            pool.rest[atomicAdd(&pool.num_rest, 1u)] = full;
+            full = kNoBatch;
+        }
+    }
+    full = __shfl_sync(kFull, full, 0);
+    __threadfence_block();
+    n = full != kNoBatch ? 32 : 0;
+    if (n) {
+        b = pool.unit[full * 32 + lane];
+        s = pool.sumsq[full * 32 + lane];
+    }
+}
+
+// After a barrier behind every warp's pool_leave(): the batch of this warp.
+// Returns its size.
+__device__ __forceinline__ int pool_rest(const EpiloguePool &pool, int32_t &b, double &s, int lane)
+{
+    const uint32_t wid = threadIdx.x >> 5, num_rest = pool.num_rest;
+    const int n = wid < num_rest ? 32 : wid == num_rest ? static_cast<int>(pool.count % 32) : 0;
+    if (lane < n) {
+        const uint32_t slot = (wid < num_rest ? pool.rest[wid] : pool.count / 32) * 32 + lane;
+        b = pool.unit[slot];
+        s = pool.sumsq[slot];
+    }
+    return n;
+}
+
 // MODE kStepFull: the whole step.  kStepPartials: phase 1 only, each unit's
 // sum of squares written to out_sumsq (the first half of a sharded step).
 // kStepFinish: no gradient read; phases 2-3 on the sums in in_sumsq (the
@@ -907,6 +986,14 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
     constexpr int kEB = Elem<DT>::kBytes;
     const int lane = threadIdx.x & 31;
     const int warp = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
+    EpiloguePool &pool = *reinterpret_cast<EpiloguePool *>(s_keys);   // until the selection, which reuses it
+    if (MODE == kStepFull && Shape<V>::kPool && p.pool) {
+        if (threadIdx.x < kWarpsPerCta)
+            pool.fill[threadIdx.x] = 0;
+        if (threadIdx.x == kWarpsPerCta)
+            pool.count = pool.warps = pool.num_rest = 0;
+        __syncthreads();
+    }
     // Launched as a programmatic dependent of whatever precedes it on the
     // stream: wait here until that kernel has completed and its writes are
     // visible (the arena, the previous step's state), then let the next step
@@ -1008,11 +1095,30 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             p.ctl->next_run = 0;
             p.ctl->warps_done = 0;
         }
-        if (MODE != kStepPartials && npend > 0)
-            unit_epilogue(p, lane < npend, pend_b, pend_s, alpha, beta, t);
+        if (MODE == kStepFull) {
+            if (Shape<V>::kPool && p.pool) {
+                const int32_t here = p.num_warps - static_cast<int32_t>(blockIdx.x) * kWarpsPerCta;   // with a first run
+                pool_leave(pool, here < kWarpsPerCta ? here : kWarpsPerCta, npend, pend_b, pend_s, lane);
+            }
+            if (npend > 0)
+                unit_epilogue(p, lane < npend, pend_b, pend_s, alpha, beta, t);
+        }
     }
     if (MODE == kStepPartials)
         return;
+
+    if (MODE == kStepFull && Shape<V>::kPool && p.pool) {
+        __syncthreads();
+        int32_t b = 0;
+        double sumsq = 0.0;
+        const int n = pool_rest(pool, b, sumsq, lane);
+        if (n > 0) {
+            const int64_t t = __ldcg(&p.ctl->steps) + 1;
+            unit_epilogue(p, lane < n, b, sumsq,
+                          pick_threshold(p.alpha_override, t, p.warmup_steps, p.alpha_init, p.alpha_main),
+                          pick_threshold(p.beta_override, t, p.warmup_steps, p.beta_init, p.beta_main), t);
+        }
+    }
 
     // Grid completion: the last CTA through runs the selection.  The barrier
     // orders the CTA's writes before thread 0's release; the last ticket's

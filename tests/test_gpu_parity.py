@@ -715,3 +715,32 @@ def test_steps_wait_for_the_kernel_that_writes_the_arena(config, shrink, cuda_de
             np.testing.assert_allclose(got[t], want, rtol=RTOL, atol=0, err_msg=f"step {t + 1}")
     finally:
         mon.close()
+
+
+@pytest.mark.parametrize("units_per_sm,extra", [(6, -1), (6, 0), (6, 1), (13, 0), (32, 1), (133, 3), (520, 0)])
+def test_pooled_epilogues_update_every_unit_once(units_per_sm, extra, cuda_device):
+    """Layouts of 6 units per SM up to 16 per warp run their last epilogue
+    batches from a pool of the CTA's units.  The controller half runs them
+    unit by unit, so both must leave the same state, masks and statistics,
+    bit for bit, on the same sums."""
+    import torch
+    U = units_per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    rng = np.random.default_rng(U)
+    lengths = rng.integers(0, 300, U).astype(np.int64)
+    offsets = np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64)
+    kw = dict(dtype="f32", window=3, max_o=7, lock_len=2, alpha=1.1, beta=1.2)
+    one, two = Monitor(offsets, lengths, **kw), Monitor(offsets, lengths, **kw)
+    try:
+        for step in range(5):
+            g = torch.Generator(cuda_device).manual_seed(step)
+            arena = torch.randn(int(lengths.sum()), device=cuda_device, generator=g) * (1.0 + (step == 4))
+            s1, s2 = one.new_stats(), two.new_stats()
+            m1 = one.step(arena, stats=s1)
+            m2 = two.finish(two.step_partials(arena), stats=s2)
+            assert torch.equal(m1, m2)
+            for key in s1:
+                assert torch.equal(s1[key], s2[key]), key
+        assert one.get_state() == two.get_state()
+    finally:
+        one.close()
+        two.close()
