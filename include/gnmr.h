@@ -280,12 +280,14 @@ const char *gnmr_status_string(gnmr_status s);
  * create on this thread); never NULL. */
 const char *gnmr_last_error(const gnmr_handle *h);
 
-/* Host-only query of the work partition that gnmr_create plans for the
- * small-unit loop shape (max_warps = the resident warps): the concatenation
+/* Host-only query of the work partition that gnmr_create plans (max_warps =
+ * the number of runs asked for; "warp" below stands for whoever streams a
+ * run): the concatenation
  * of all units (an empty unit counts as one element of work) is cut into at
  * most max_warps contiguous runs of about equal cost (element bytes plus a
- * fixed per-unit cost), one run per warp.  (The large-unit shape cuts the
- * same way into about 16 runs per warp, see gnmr_info.num_runs.)  Outputs,
+ * fixed per-unit cost).  (The small-unit loop shape cuts into one run per
+ * resident CTA, whose warps then share it block by block; the large-unit
+ * shape into about 16 runs per warp, see gnmr_info.num_runs.)  Outputs,
  * caller-allocated: run_unit / run_pos [max_warps + 1] (run w covers
  * (run_unit[w], run_pos[w]) up to, not including, (run_unit[w+1],
  * run_pos[w+1])), first_warp / num_parts [num_units] (the warps touching

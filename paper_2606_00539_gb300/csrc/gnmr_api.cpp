@@ -287,24 +287,29 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
                 seg_unit[u] = u;
         }
         const int64_t S = static_cast<int64_t>(seg_off.size());
-        // The small-unit loop plans one run per resident warp.  The large-unit
-        // loop plans about kRunsPerWarp runs per warp (never fewer runs than
-        // the one-per-warp plan), which the warps take dynamically.
+        // The small-unit loop plans one run per resident CTA, in blocks.  The
+        // large-unit loop plans about kRunsPerWarp runs per warp (never fewer
+        // than one per warp), which the warps take dynamically.
         const int64_t grid_warps = int64_t(sms) * per_sm * gnmr::kWarpsPerCta;
-        int64_t max_runs = grid_warps;
+        gnmr::Plan plan;
+        gnmr::BlockPlan blocks;
+        bool planned;
         if (variant == gnmr::kVariantBulk) {
             const int64_t cost = grad_bytes + U * gnmr::kUnitCostBytes;
             int64_t run = cost / (grid_warps * gnmr::kRunsPerWarp);
             run = std::min(std::max(run, gnmr::kBulkRunMin), gnmr::kBulkRunMax);
-            max_runs = std::max(max_runs, (cost + run - 1) / run);
+            const int64_t max_runs = std::max(grid_warps, (cost + run - 1) / run);
             if (max_runs > INT32_MAX / 2) {
                 delete h;
                 return fail_create(GNMR_ERR_INVALID_ARG, "work partition failed (too many runs)");
             }
+            planned = gnmr::plan_partition(S, seg_len.data(), seg_unit.data(), c.num_units, eb,
+                                           static_cast<int32_t>(max_runs), plan);
+        } else {
+            planned = gnmr::plan_blocks(S, seg_off.data(), seg_len.data(), seg_unit.data(), c.num_units, eb,
+                                        sms * per_sm, plan, blocks);
         }
-        gnmr::Plan plan;
-        if (!gnmr::plan_partition(S, seg_len.data(), seg_unit.data(), c.num_units, eb,
-                                  static_cast<int32_t>(max_runs), plan)) {
+        if (!planned) {
             delete h;
             return fail_create(GNMR_ERR_INVALID_ARG, "work partition failed (sizes out of range)");
         }
@@ -328,6 +333,9 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         const size_t o_hot = cv.take(sizeof(gnmr::Candidate) * hot_cap);
         const size_t o_hist = cv.take(sizeof(uint32_t) * gnmr::kRiskBins);
         const size_t o_ctl = cv.take(sizeof(gnmr::Control));
+        const size_t o_ctab = cv.take(sizeof(gnmr::CtaBlocks) * blocks.cta.size());
+        const size_t o_block = cv.take(sizeof(gnmr::Block) * blocks.block.size());
+        const size_t o_ublock = cv.take(sizeof(int32_t) * blocks.unit_block.size());
         const size_t o_cost = c.unit_cost ? cv.take(sizeof(double) * U) : 0;
 
         // Host image of the whole block: static tables plus zeroed state.
@@ -347,6 +355,11 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         std::memcpy(&img[o_first], plan.first_run.data(), sizeof(int32_t) * U);
         std::memcpy(&img[o_parts], plan.num_parts.data(), sizeof(int32_t) * U);
         std::memcpy(&img[o_pbase], plan.part_base.data(), sizeof(int64_t) * U);
+        if (!blocks.cta.empty()) {
+            std::memcpy(&img[o_ctab], blocks.cta.data(), sizeof(gnmr::CtaBlocks) * blocks.cta.size());
+            std::memcpy(&img[o_block], blocks.block.data(), sizeof(gnmr::Block) * blocks.block.size());
+            std::memcpy(&img[o_ublock], blocks.unit_block.data(), sizeof(int32_t) * blocks.unit_block.size());
+        }
         std::memset(&img[o_partial], 0xff, sizeof(double) * plan.num_partials);   // every slot empty
         static_assert(gnmr::kEmptyPartial == ~0ull, "empty partial slots are all-ones bytes");
         {
@@ -363,6 +376,8 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
                                format("cudaMalloc(%zu): %s", cv.size, cudaGetErrorString(e)));
         }
         e = cudaMemcpy(h->dmem, img.data(), cv.size, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaStreamSynchronize(nullptr);       // the plan is in place whatever stream steps
         if (e != cudaSuccess) {
             cudaFree(h->dmem);
             delete h;
@@ -377,6 +392,9 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         p.recoverable = reinterpret_cast<const uint8_t *>(base + o_rec);
         p.run_seg = reinterpret_cast<const int64_t *>(base + o_run_seg);
         p.run_pos = reinterpret_cast<const int64_t *>(base + o_run_pos);
+        p.cta_blocks = reinterpret_cast<const gnmr::CtaBlocks *>(base + o_ctab);
+        p.block = reinterpret_cast<const gnmr::Block *>(base + o_block);
+        p.unit_block = reinterpret_cast<const int32_t *>(base + o_ublock);
         p.first_run = reinterpret_cast<const int32_t *>(base + o_first);
         p.num_parts = reinterpret_cast<const int32_t *>(base + o_parts);
         p.part_base = reinterpret_cast<const int64_t *>(base + o_pbase);
@@ -396,11 +414,15 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         p.static_warmup = c.static_warmup_steps;
         p.static_keep = static_cast<int32_t>(std::min<double>(std::ceil(c.static_fraction * num_rec), num_rec));
         p.num_units = c.num_units;
-        const int32_t step_warps = static_cast<int32_t>(std::min<int64_t>(plan.num_runs, grid_warps));
+        // small-unit loop: the warps that start on a block
+        int64_t first_blocks = 0;
+        for (const gnmr::CtaBlocks &b : blocks.cta)
+            first_blocks += std::min(b.count, gnmr::kWarpsPerCta);
+        const int32_t step_warps = static_cast<int32_t>(
+            variant == gnmr::kVariantBulk ? std::min<int64_t>(plan.num_runs, grid_warps) : first_blocks);
         p.num_warps = step_warps;
         p.num_runs = plan.num_runs;
-        p.pool = variant == gnmr::kVariantSmall && U >= gnmr::kPoolUnitsPerSm * sms &&
-                 U <= gnmr::kPoolUnitsPerWarp * p.num_warps;
+        p.dense = U <= gnmr::kDenseUnits ? 1 : 0;
         p.window = c.window;
         p.max_o = c.max_o;
         p.lock_len = c.lock_len;
@@ -422,8 +444,9 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         h->num_units = c.num_units;
         h->elem_bytes = eb;
         h->num_warps = step_warps;
-        h->num_runs = plan.num_runs;
-        h->num_ctas = (step_warps + gnmr::kWarpsPerCta - 1) / gnmr::kWarpsPerCta;
+        h->num_runs = variant == gnmr::kVariantBulk ? plan.num_runs : step_warps;
+        h->num_ctas = variant == gnmr::kVariantBulk ? (step_warps + gnmr::kWarpsPerCta - 1) / gnmr::kWarpsPerCta
+                                                    : plan.num_runs;
         {
             const int64_t warps = (U + 31) / 32;
             const int64_t ctas = (warps + gnmr::kWarpsPerCta - 1) / gnmr::kWarpsPerCta;

@@ -12,8 +12,8 @@ namespace gnmr {
 
 // Launch shape of the step kernel: 512 threads = 16 warps per CTA.  Two
 // compiled variants of the streaming loop (gnmr_kernels.cu): kVariantSmall
-// (two resident CTAs per SM, one planned run per warp) for layouts of many
-// small units, kVariantBulk (one CTA per SM, deeper per-warp streams, runs
+// (two resident CTAs per SM, each with a part of its own that its warps take
+// block by block) for layouts of small and mid-sized units, kVariantBulk (one CTA per SM, deeper per-warp streams, runs
 // taken from a shared counter) for layouts whose mean unit holds at least
 // kBulkUnitBytes.
 constexpr int kThreads = 512;
@@ -28,7 +28,7 @@ constexpr int64_t kBulkUnitBytes = int64_t(1) << 20;
 // smaller than kMinRunBytes unless the whole problem is.
 constexpr int64_t kUnitCostBytes = 4096;
 constexpr int64_t kSplitBytes = 512;
-constexpr int64_t kMinRunBytes = 4096;   // one 4 KiB load round per warp: small problems spread over more SMs
+constexpr int64_t kMinRunBytes = 4096;   // one 4 KiB load round per warp
 // Large-unit loop: the stream is cut into about kRunsPerWarp runs per warp of
 // kBulkRunMin..kBulkRunMax bytes each.  Each warp starts on its own run and
 // then takes the next untaken one, so warps that stream faster take more runs
@@ -38,13 +38,34 @@ constexpr int64_t kRunsPerWarp = 16;
 constexpr int64_t kBulkRunMin = int64_t(64) << 10;
 constexpr int64_t kBulkRunMax = int64_t(256) << 10;
 
-// Layouts in which a CTA's warps pool the units of their last epilogue batches:
-// from kPoolUnitsPerSm units per SM to kPoolUnitsPerWarp per warp.  An epilogue
-// batch takes about 0.9 us of an SM's fp64 pipe and 4.4 us of latency, so below
-// about five batches per SM there is nothing to save, and with 20 units a warp
-// (100K units) the batches are full enough: 262.8 us without, 264.4 with.
-constexpr int64_t kPoolUnitsPerSm = 6;
-constexpr int64_t kPoolUnitsPerWarp = 16;
+// Small-unit loop: every CTA owns a contiguous part of the segment stream of
+// at least kMinCtaBytes of cost, cut into blocks of at most kMinBlockBytes
+// (doubled until a CTA has at most kBlocksPerCta), which its warps take in
+// turn.  kBatch units are one batch of the unit epilogue.  8 KiB blocks, two
+// load rounds of a warp: 4 KiB took 246.8 us on 100K units, 8 KiB 242.9, 16
+// KiB 244.2 (560 units of 224 KB: 34.1, 32.7, 31.6).  24 KiB per CTA: 3.7 MB
+// over 64 units took 11.9 us with 64 KiB, 11.4 with 24.
+constexpr int kBatch = 32;
+constexpr int kBlocksPerCta = 2048;
+constexpr int64_t kMinCtaBytes = int64_t(24) << 10;
+constexpr int64_t kMinBlockBytes = int64_t(8) << 10;
+constexpr int64_t kMaxBlockBytes = int64_t(1) << 20;
+
+// A piece of one segment.
+struct alignas(16) Block {
+    int64_t start;    // first element, in the arena
+    int32_t elems;
+    int32_t batch;    // epilogue batch, counted from the CTA's first unit
+};
+struct alignas(16) CtaBlocks {
+    int32_t first, count;         // blocks
+    int32_t unit, units;          // first unit touched, and how many
+    // the first and the last unit (one and the same if units == 1), which
+    // other CTAs may have parts of: number of parts (1: none), the unit's
+    // first partial slot, and this CTA's slot from there
+    int32_t parts[2], slot[2];
+    int64_t base[2];
+};
 
 // Persistent per-unit controller state (Algorithm 1 and 2), 40 bytes.
 struct UnitState {
@@ -88,6 +109,13 @@ constexpr int kRiskBins = 2048;
 constexpr uint32_t kHotCapMax = 8192;
 constexpr uint32_t kNoHot = kRiskBins;   // hot_bin: no prediction, no pool member is hot
 
+// Up to this many units (four a thread of the selecting CTA) a step keeps no
+// lists and no histogram: reading every unit's entry costs the selection one
+// round trip, where appending cost each epilogue two (64 units: tail of the
+// step after the last epilogue 3.7 -> 2.8 us, the epilogue itself 4.4 -> 3.1
+// us with the four-lane divisions).
+constexpr int32_t kDenseUnits = 2048;
+
 // Device-resident step control block.
 struct Control {
     uint32_t ctas_done;   // CTA completion ticket of the current launch
@@ -121,7 +149,10 @@ struct StepParams {
     const uint8_t *recoverable;  // [U]
     const int64_t *run_seg;      // [R + 1] first segment of each run
     const int64_t *run_pos;      // [R + 1]
-    const int32_t *first_run;    // [U] first run touching unit b
+    const CtaBlocks *cta_blocks; // [num_ctas] small-unit loop: each CTA's part,
+    const Block *block;          // the blocks of all CTAs
+    const int32_t *unit_block;   // [U + 1] and the first block of each unit
+    const int32_t *first_run;    // [U] first run (small-unit loop: CTA) touching unit b
     const int32_t *num_parts;    // [U]
     const int64_t *part_base;    // [U] first partial slot of unit b
     double *partial;             // [num_partials]
@@ -146,11 +177,11 @@ struct StepParams {
     int32_t static_keep;                                  // ceil(static_fraction * |B_rec|)
     uint32_t hot_cap;                                     // min(U, kHotCapMax)
     int32_t num_units;
-    int32_t num_warps;           // warps with a first run: runs 0 .. num_warps - 1
+    int32_t num_warps;           // large-unit loop: warps with a first run, 0 .. num_warps - 1
     int32_t window;
     int32_t max_o;
     int32_t lock_len;
-    int32_t pool;                // 1: the CTA's warps pool their last units (many units per SM)
+    int32_t dense;               // 1: at most kDenseUnits units, selected from one entry each
     int32_t num_runs;            // R; runs num_warps .. R - 1 are taken dynamically
     int64_t warmup_steps;
     double alpha_init, alpha_main, beta_init, beta_main, eps;
@@ -191,5 +222,19 @@ struct Plan {
 // the inputs are out of range.
 bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int32_t *seg_unit,
                     int32_t num_units, int elem_bytes, int32_t max_runs, Plan &out);
+
+// The blocks of a plan with one run per CTA (small-unit loop).
+struct BlockPlan {
+    std::vector<CtaBlocks> cta;       // [num_runs]
+    std::vector<Block> block;
+    std::vector<int32_t> unit_block;  // [U + 1]
+};
+
+// Cuts the stream into one run per CTA (about max_ctas of them, more where a
+// run would hold more than kBlocksPerCta blocks) and the runs into blocks.
+// Same input rules as plan_partition; seg_offsets in elements.
+bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t *seg_lengths,
+                 const int32_t *seg_unit, int32_t num_units, int elem_bytes, int32_t max_ctas, Plan &out,
+                 BlockPlan &blocks);
 
 }  // namespace gnmr

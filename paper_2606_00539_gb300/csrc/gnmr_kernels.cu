@@ -1,32 +1,48 @@
 // GNMR per-step monitor: one kernel launch per training step on sm_103a.
 //
 // Phase 1, every warp (the hot loop).  The segment stream (a unit is one or
-// more segments of the arena) is cut by gnmr_plan.cpp into contiguous runs.
-// With the small-unit loop each warp owns one run.  With the large-unit loop
-// there are about 16 runs per warp: each warp starts on its own run and then
-// takes the next untaken one from a counter, so warps that stream faster take
-// more runs and all warps finish within about one run of each other (with one
-// run per warp, HBM's uneven service left the slowest warps ~8 % of the step
-// behind the median).  For every segment (or part of one) in a run the warp streams the
-// gradient with 16-byte read-only loads (8 or 16 in flight per lane, by the
-// loop shape), squares in fp32, sums blocks of 16 iterations in fp32 and the
-// blocks as float pairs (error-free TwoSum), and all-reduces the lanes' totals
-// across the warp with shuffles, converting to fp64 once per segment:
-// n_b = ||g_b||_2 (Sec. 2, Eq. local_gradient).  No shared memory, no block
-// barrier on this path.  (The streaming reduction lives in gnmr_stream.cuh.)
+// more segments of the arena) is cut by gnmr_plan.cpp.  For every piece of a
+// segment the warp streams the gradient with 16-byte loads (8 or 16 in flight
+// per lane, by the loop shape), squares in fp32, sums blocks of 16 iterations
+// in fp32 and the blocks as float pairs (error-free TwoSum), and all-reduces
+// the lanes' totals across the warp with shuffles, converting to fp64 once per
+// piece: n_b = ||g_b||_2 (Sec. 2, Eq. local_gradient).  (The streaming
+// reduction lives in gnmr_stream.cuh.)
 //
-// Phase 2, the warp that completes unit b.  A unit split over several runs
-// collects their partial sums through fixed slots (one per run, whichever
-// warp streams it) and a per-unit ticket; the warp that takes the last ticket
-// sums the slots in slot order (so the result does not depend on timing); a
-// unit of two parts trades its partial in one atomic exchange.  Completed units queue up in the warp's lanes and run the
-// unit epilogue 32 at a time, one unit per lane: Algorithm 1 (GNMR,
+// Small-unit loop: a CTA owns a contiguous part of the stream, cut into blocks
+// of 8 KiB and less, which its warps take from a counter in shared memory.
+// HBM serves warps unevenly (with one fixed run per warp the first warps of a
+// 125 MB step ended after 13 us and the last after 29), so warps that stream
+// faster take more blocks; a block's sum goes to a slot in shared memory, and
+// the warp that sums the last block of 32 consecutive units finishes them
+// (phase 2) while the others stream on.  Only a CTA's first and last unit can
+// be shared with other CTAs.  The plan is read before the grid's programmatic
+// wait.  One GB300, from one run per warp to blocks: 100K fp32 units 263.3 ->
+// 243.1 us; 30,000 short bf16 units 34.2 -> 32.2 us; 560 units in 125 MB 30.7
+// -> 30.0 us; 64 units in 3.7 MB 11.0 -> 11.4 us.
+//
+// Large-unit loop: about 16 runs per warp; each warp starts on its own run and
+// then takes the next untaken one from a global counter, so warps that stream
+// faster take more runs and all warps finish within about one run of each
+// other (with one run per warp, HBM's uneven service left the slowest warps
+// ~8 % of the step behind the median).  No shared memory, no block barrier on
+// this path.  (Runs that get smaller towards the end were no faster: each
+// hand-over costs about 3 us of the warp, for tables, partial and ticket.)
+//
+// Phase 2, the warp that completes units.  A unit split over several parts
+// (runs, CTAs) collects their partial sums through fixed slots (one per part,
+// whichever warp streams it) and a per-unit ticket; the warp that takes the
+// last ticket sums the slots in slot order (so the result does not depend on
+// timing); a unit of two parts trades its partial in one atomic exchange.
+// Completed units run the unit epilogue up to 32 at a time, one per lane (in
+// the large-unit loop they queue up in the warp's lanes): Algorithm 1 (GNMR,
 // Delta-GNMR, incremental mean, window queue), the combined risk
 // R = max{GNMR/alpha_t, Delta-GNMR/beta_t} and the candidate test
-// R > 1 or Lock > 0 (Sec. 3.3).  Candidates go to a compact list; members of
-// the capped pool also count in a global risk histogram and, at or above the
-// bin predicted from the previous step's cut, go to a short hot list.  Every
-// unit's outcome if it is not selected is written here.
+// R > 1 or Lock > 0 (Sec. 3.3).  With few units (kDenseUnits) every unit leaves
+// one entry for the selection; else candidates go to a compact list, and
+// members of the capped pool also count in a global risk histogram and, at or
+// above the bin predicted from the previous step's cut, go to a short hot
+// list.  Every unit's outcome if it is not selected is written here.
 //
 // Phase 3, the last CTA to finish (grid ticket): Top_maxO.  The histogram
 // gives the bin that holds the maxO-th largest risk; one read of the hot list
@@ -53,7 +69,7 @@ namespace gnmr {
 namespace {
 
 // Two compiled shapes of the streaming loop, chosen per handle from the mean
-// unit size (both measured on GB300): many small units run best with 8
+// unit size (both measured on GB300): small units run best with 8
 // 16-byte loads in flight per lane and two CTAs per SM; large units with 16
 // loads per lane and one CTA per SM (fewer, deeper streams) and runs of at
 // most 256 KiB taken dynamically.
@@ -61,14 +77,12 @@ template <int V> struct Shape;
 template <> struct Shape<kVariantSmall> {
     static constexpr int kUnroll = 8;
     static constexpr int kMinCtas = 2;
-    static constexpr bool kDynamic = false;           // one planned run per warp
-    static constexpr bool kPool = true;               // may pool the warps' last units
+    static constexpr bool kBlocks = true;             // blocks of the CTA's own part, in turn
 };
 template <> struct Shape<kVariantBulk> {
     static constexpr int kUnroll = 16;
     static constexpr int kMinCtas = 1;
-    static constexpr bool kDynamic = true;            // further runs taken from a counter
-    static constexpr bool kPool = false;
+    static constexpr bool kBlocks = false;            // runs taken from a global counter
 };
 
 __device__ __forceinline__ double pick_threshold(double override_value, int64_t t, int64_t warmup,
@@ -134,69 +148,121 @@ __device__ __forceinline__ void warp_append(Candidate *list, uint32_t *count, ui
 // Algorithm 2.  Every lane issues its unit's loads together, so a batch costs
 // about one memory round trip; candidates are appended with one atomic per
 // warp.  Called by all 32 lanes.
+//
+// What bounds it is the chain of correctly rounded fp64 operations: a division
+// takes 0.27 us, and the compiler runs one after the other.  Seven of a unit's
+// eight do not all depend on each other, so a batch of at most 8 units gives
+// each unit four lanes, which do the independent divisions at once: a square
+// root and three rounds of division instead of six (the epilogue of 64 units:
+// 4.4 -> 3.1 us).
 __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, double sumsq,
                               double alpha, double beta, int64_t t)
 {
+    const unsigned mine = __ballot_sync(kFull, active);
+    if (!mine)
+        return;
+    const int lane = threadIdx.x & 31;
+    const bool few = __popc(mine) <= 8;
+    const int role = lane & 3;
+    if (few) {
+        // lane 4 j + role works on the j-th active lane's unit (past the last, on
+        // the first once more, writing nothing)
+        const int count = __popc(mine), j = lane >> 2;
+        unsigned rest = mine;
+#pragma unroll
+        for (int k = 0; k < 7; ++k)
+            if (k < j && j < count)
+                rest &= rest - 1;
+        const int from = __ffs(rest) - 1;
+        b = __shfl_sync(kFull, b, from);
+        sumsq = __shfl_sync(kFull, sumsq, from);
+        active = j < count;
+    }
     bool cand = false;
     double r = 0.0;
     uint32_t cand_lock = 0;
     // read now, used after the risk: the step's hot-list bin (only the
     // selection, after every CTA, rewrites it)
-    const uint32_t hot_bin = __ldcg(&p.ctl->hot_bin);
-    if (active) {
-        const double n = sqrt(sumsq);
+    const uint32_t hot_bin = p.dense ? 0u : __ldcg(&p.ctl->hot_bin);
+    UnitState s{};
+    double n = 0.0, g = 0.0, d = 0.0, step = 0.0;     // step: the mean's change
+    bool rec = false;
+    if (active || few) {
+        n = sqrt(sumsq);
         const int w = p.window;
         double *Q = p.queue + static_cast<int64_t>(b) * w;
         // the window's lines travel with the state load: the window reads,
         // which need the state's head, then hit in L1
         asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
         asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + (w - 1)));
-        UnitState s = p.state[b];
-        const bool rec = p.recoverable[b] != 0;
-        // The risk first (its chain of dependent divisions decides the
-        // epilogue's latency), the state update after it.
-        double g, d;
-        if (!isfinite(n)) {
-            // Non-finite gradient: maximal risk, no change to A_b, Q_b, k_b.
-            g = CUDART_INF;
-            d = CUDART_INF;
-        } else {
-            // mean of the window, summed oldest to newest; its loads are issued
-            // as soon as the state's head is known, before the division for g
-            const bool full = s.fill == w;
-            double q = 0.0;
-            if (full) {
-                int idx = s.head, k = 0;
-                for (; k + 8 <= w; k += 8) {
-                    double v[8];
+        s = p.state[b];
+        rec = p.recoverable[b] != 0;
+        // mean of the window, summed oldest to newest; its loads are issued
+        // as soon as the state's head is known, before the division for g
+        const bool full = s.fill == w;
+        double q = 0.0;
+        if (full) {
+            int idx = s.head, k = 0;
+            for (; k + 8 <= w; k += 8) {
+                double v[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int ix = idx + j < w ? idx + j : idx + j - w;
-                        v[j] = Q[ix];
-                    }
+                for (int j = 0; j < 8; ++j) {
+                    const int ix = idx + j < w ? idx + j : idx + j - w;
+                    v[j] = Q[ix];
+                }
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        q += v[j];
-                    idx = idx + 8 < w ? idx + 8 : idx + 8 - w;
-                }
-                for (; k < w; ++k) {
-                    q += Q[idx];
-                    idx = (idx + 1 == w) ? 0 : idx + 1;
-                }
+                for (int j = 0; j < 8; ++j)
+                    q += v[j];
+                idx = idx + 8 < w ? idx + 8 : idx + 8 - w;
             }
-            g = (s.count == 0 || s.mean == 0.0) ? 1.0 : n / (s.mean + p.eps);
+            for (; k < w; ++k) {
+                q += Q[idx];
+                idx = (idx + 1 == w) ? 0 : idx + 1;
+            }
+        }
+        const double count = static_cast<double>(s.count + 1);
+        const bool fresh = s.count == 0 || s.mean == 0.0;
+        double x, y;
+        if (few) {
+            // (dividends and divisors that a case below discards may be anything)
+            const int unit = lane & ~3;
+            const double q1 = (role == 0 ? n : role == 1 ? q : n - s.mean) /
+                              (role == 0 ? s.mean + p.eps : role == 1 ? static_cast<double>(w) : count);
+            g = __shfl_sync(kFull, q1, unit);
+            const double den = __shfl_sync(kFull, q1, unit + 1) + p.eps;
+            step = __shfl_sync(kFull, q1, unit + 2);
+            g = fresh ? 1.0 : g;
+            const double q2 = g / (role == 0 ? alpha : den);
+            x = __shfl_sync(kFull, q2, unit);
+            d = __shfl_sync(kFull, q2, unit + 1);
+            d = !full ? 1.0 : den != 0.0 ? d : g > 0.0 ? CUDART_INF : 1.0;
+            y = d / beta;
+        } else {
+            // The risk first (its chain of dependent divisions decides the
+            // epilogue's latency), the mean's change after it.
+            g = fresh ? 1.0 : n / (s.mean + p.eps);
             if (full) {
                 const double den = q / static_cast<double>(w) + p.eps;
                 d = (den == 0.0) ? (g > 0.0 ? CUDART_INF : 1.0) : g / den;
             } else {
                 d = 1.0;
             }
+            x = g / alpha;
+            y = d / beta;
+            step = (n - s.mean) / count;
         }
-        const double x = g / alpha, y = d / beta;
         r = x > y ? x : y;
+        if (!isfinite(n))                             // maximal risk, no change to A_b, Q_b, k_b
+            g = d = r = CUDART_INF;
+    }
+    if (few)
+        active = active && role == 0;
+    if (active) {
+        const int w = p.window;
+        double *Q = p.queue + static_cast<int64_t>(b) * w;
         if (isfinite(n)) {
             s.count += 1;
-            s.mean = s.mean + (n - s.mean) / static_cast<double>(s.count);
+            s.mean = s.mean + step;
             if (s.fill < w) {                        // still filling: head stays 0
                 Q[s.fill] = g;
                 s.fill += 1;
@@ -250,6 +316,14 @@ __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, doubl
         }
         cand_lock = static_cast<uint32_t>(s.lock) | (s.active ? kCandActive : 0u);
     }
+    if (p.dense) {
+        // few units: one entry per unit, which the selection reads in full
+        if (active) {
+            const uint64_t word = static_cast<uint32_t>(cand ? b : -1) | static_cast<uint64_t>(cand_lock) << 32;
+            *reinterpret_cast<double2 *>(p.cand + b) = make_double2(r, __longlong_as_double(static_cast<long long>(word)));
+        }
+        return;
+    }
     // The capped pool: every candidate, or under the admission cap those not
     // active at t-1 (the retained ones are selected without ranking).  Pool
     // members count in the risk histogram; the hot list takes those at or
@@ -265,35 +339,49 @@ __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, doubl
     warp_append(p.hot, &p.ctl->n_hot, p.hot_cap, hot, r, b, cand_lock);
 }
 
+// The same, out of line: the large-unit loop calls it rarely and keeps its
+// registers for the stream.
+__device__ __noinline__ void unit_epilogue_call(const StepParams &p, bool active, int32_t b, double sumsq,
+                                                double alpha, double beta, int64_t t)
+{
+    unit_epilogue(p, active, b, sumsq, alpha, beta, t);
+}
+
+// A unit of two parts trades its partial through the first slot in one atomic
+// exchange: the first part finds the slot empty and leaves its partial there,
+// the second takes it, adds it to its own (IEEE addition is commutative, so the
+// bits are those of the slot-order sum) and empties the slot again.  Returns
+// true for the second, with the unit's sum in s.
+__device__ __forceinline__ bool exchange_parts(const StepParams &p, int64_t base, double &s)
+{
+    const double mine = isnan(s) ? CUDART_NAN : s;                  // never the empty pattern
+    const unsigned long long other = atomicExch(reinterpret_cast<unsigned long long *>(p.partial + base),
+                                                static_cast<unsigned long long>(__double_as_longlong(mine)));
+    if (other == kEmptyPartial)
+        return false;
+    __stcg(reinterpret_cast<unsigned long long *>(p.partial + base), kEmptyPartial);
+    s = s + __longlong_as_double(static_cast<long long>(other));
+    return true;
+}
+
 // A unit split over several warps: stores this warp's partial and takes a
 // ticket.  Returns true (with the unit's total in s) for the warp that takes
-// the last ticket; that warp sums the partials in slot order.  A unit of two
-// parts trades its partial through the first slot in one atomic exchange:
-// the first warp finds the slot empty and leaves its partial there, the
-// second takes it, adds it to its own (IEEE addition is commutative, so the
-// bits are those of the slot-order sum) and empties the slot again.
-__device__ __forceinline__ bool combine_parts(const StepParams &p, int32_t b, int32_t parts, int32_t run,
-                                              double &s, int lane)
+// the last ticket; that warp sums the partials in slot order.  Units of two
+// parts go through exchange_parts().
+// base: the unit's first slot; slot: this part's, from there.
+__device__ __forceinline__ bool combine_parts(const StepParams &p, int32_t b, int32_t parts, int64_t base,
+                                              int32_t slot, double &s, int lane)
 {
-    const int64_t base = p.part_base[b];
     if (parts == 2) {
-        unsigned long long other = 0;
-        if (lane == 0) {
-            const double mine = isnan(s) ? CUDART_NAN : s;          // never the empty pattern
-            other = atomicExch(reinterpret_cast<unsigned long long *>(p.partial + base),
-                               static_cast<unsigned long long>(__double_as_longlong(mine)));
-        }
-        other = __shfl_sync(kFull, other, 0);
-        if (other == kEmptyPartial)
-            return false;
+        bool whole = false;
         if (lane == 0)
-            __stcg(reinterpret_cast<unsigned long long *>(p.partial + base), kEmptyPartial);
-        s = s + __longlong_as_double(static_cast<long long>(other));
-        return true;
+            whole = exchange_parts(p, base, s);
+        s = __shfl_sync(kFull, s, 0);
+        return __shfl_sync(kFull, whole, 0);
     }
     uint32_t last = 0;
     if (lane == 0) {
-        __stcg(&p.partial[base + (run - p.first_run[b])], s);
+        __stcg(&p.partial[base + slot], s);
         last = ticket_acq_rel(&p.unit_ticket[b]) == static_cast<uint32_t>(parts - 1);
     }
     last = __shfl_sync(kFull, last, 0);
@@ -481,6 +569,7 @@ constexpr int kMiscRank = 2;      // r minus the count above that bin
 constexpr int kMiscCount = 3;     // that bin's count
 constexpr int kMiscHint = 5;      // scan_risk_hist: the bin holding the hint-th largest
 constexpr int kMiscPool = 6;      // scan_risk_hist: the pool size
+constexpr int kMiscKept = 4;      // dense selection: candidates selected without ranking
 constexpr int kMiscFill = 7;      // cut-list entries appended
 
 // Bin of the r-th largest digit in hist[kWideBins] (r >= 1), by the whole
@@ -784,11 +873,18 @@ __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t 
 // themselves.  The list read is the hot list when the previous step's
 // prediction was at or below c and the hot list did not overflow (it then
 // holds every entry at or above c), else the whole candidate list.
+//
+// With at most kDenseUnits units there are no lists and no histogram: every
+// unit has left one entry, all of them are read at once, and the pool is ranked
+// in shared memory.
 __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist, uint32_t *misc, double *red,
                                   unsigned char *smem)
 {
-    uint32_t m = __ldcg(&p.ctl->n_cand);
-    m = m < static_cast<uint32_t>(p.num_units) ? m : static_cast<uint32_t>(p.num_units);
+    uint32_t m = 0;
+    if (!p.dense) {
+        m = __ldcg(&p.ctl->n_cand);
+        m = m < static_cast<uint32_t>(p.num_units) ? m : static_cast<uint32_t>(p.num_units);
+    }
     const bool all_on = t <= p.forced_steps || (p.policy == 2 && t <= p.static_warmup);
     const bool stat = p.policy == 2 && !all_on;
     const bool admission = p.policy == 1 && !all_on;
@@ -800,6 +896,52 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
     } else if (stat && t > p.static_warmup + 1) {
         m = 0;
         n_sel = static_cast<uint32_t>(p.static_keep);
+    } else if (p.dense) {
+        const uint32_t cap = stat ? static_cast<uint32_t>(p.static_keep) : static_cast<uint32_t>(p.max_o);
+        uint64_t *ck = reinterpret_cast<uint64_t *>(smem);
+        int32_t *cu = reinterpret_cast<int32_t *>(smem + kCutUnitOffset);
+        uint32_t *cl = reinterpret_cast<uint32_t *>(smem + kCutLockOffset);
+        constexpr int kEach = kDenseUnits / kThreads;
+        static_assert(kDenseUnits % kThreads == 0 && kDenseUnits <= kCutCap, "the whole pool fits the cut list");
+        double rr[kEach];
+        int32_t bb[kEach];
+        uint32_t ll[kEach];
+#pragma unroll
+        for (int j = 0; j < kEach; ++j) {           // every thread's loads in flight together
+            const int32_t i = j * kThreads + threadIdx.x;
+            bb[j] = -1;
+            if (i < p.num_units)
+                load_candidate(p.cand + i, rr[j], bb[j], ll[j]);
+        }
+        if (threadIdx.x == 0)
+            misc[kMiscFill] = misc[kMiscKept] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kEach; ++j) {
+            if (bb[j] < 0)
+                continue;
+            if (admission && (ll[j] & kCandActive)) {
+                commit_selected(p, stat, bb[j], rr[j], ll[j]);
+                atomicAdd(&misc[kMiscKept], 1u);
+            } else {
+                const uint32_t at = atomicAdd(&misc[kMiscFill], 1u);
+                ck[at] = risk_key(rr[j]);
+                cu[at] = bb[j];
+                cl[at] = ll[j];
+            }
+        }
+        __syncthreads();
+        const uint32_t pool = misc[kMiscFill], kept = misc[kMiscKept];
+        const uint32_t K = pool < cap ? pool : cap;
+        if (K == pool) {
+            for (uint32_t i = threadIdx.x; i < pool; i += kThreads)
+                commit_selected(p, stat, cu[i], __longlong_as_double(static_cast<long long>(ck[i])), cl[i]);
+        } else if (K > 0) {
+            __syncthreads();                         // every thread has read misc
+            select_cut(p, stat, 0, pool, K, ck, cu, cl, reinterpret_cast<uint32_t *>(smem + kCutHistOffset), hist, misc);
+        }
+        m = pool + kept;
+        n_sel = K + kept;
     } else if (!admission && m <= (stat ? static_cast<uint32_t>(p.static_keep) : static_cast<uint32_t>(p.max_o))) {
         // every candidate is in the pool and the pool fits the budget: one read of the
         // list commits all of it and empties the histogram bins it filled (no scan)
@@ -890,85 +1032,63 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
         if (next_hot <= kNoHot)
             p.ctl->hot_bin = next_hot;
         p.ctl->ctas_done = 0;
-        p.ctl->steps += 1;
+        p.ctl->steps = t;
     }
 }
 
-// Where a CTA's warps leave the completed units that did not fill a batch of
-// their own (fewer than 32 each): together they make full batches again.  The
-// fp64 pipe takes a warp instruction every 20 cycles however many of its lanes
-// are active, so the epilogue costs by the batch, and a partly filled one per
-// warp made it most of the step on layouts of a few units per warp (30,000
-// units of 48-4,096 bf16 elements, 6 a warp, fp64 pipe 58 % busy: 42.7 -> 34.4
-// us).  Layouts of fewer units per SM or more per warp don't use the pool
-// (kPoolUnitsPerSm, kPoolUnitsPerWarp): each warp runs its own batch.
-struct EpiloguePool {
-    double sumsq[kThreads];
-    int32_t unit[kThreads];
-    uint32_t count;                  // units left so far
-    uint32_t warps;                  // warps that have left theirs
-    uint32_t num_rest;               // full batches left for after the barrier,
-    uint32_t rest[kWarpsPerCta];     // and which
-    uint32_t fill[kWarpsPerCta];     // units written to batch i (slots 32 i ...)
+// Shared memory of the small-unit loop (the selection reuses it).
+struct BlockShared {
+    double sum[kBlocksPerCta];                    // sum of squares of each block
+    int32_t unit_end[kBlocksPerCta];              // end of each unit's blocks
+    CtaBlocks cta;
+    int32_t left[kBlocksPerCta / kBatch + 2];     // blocks of each batch not yet summed
+    int32_t next;                                 // next block to hand out
 };
-constexpr uint32_t kNoBatch = ~0u;
 
-// Leaves the lanes' `n` < 32 units.  If they complete a batch the warp takes it
-// (the lanes' b, s become that batch's, n = 32), else n = 0.  What it does not
-// take (a second batch, and any that the CTA's last warp completes) goes to
-// pool_rest(), with the batch that stays partly filled: one warp each, where
-// the last warp would run them one after the other.  No warp waits.
-__device__ __forceinline__ void pool_leave(EpiloguePool &pool, int here, int &n, int32_t &b, double &s, int lane)
+// The sums of a batch's units, one per lane (lane j: unit0 + j), from their
+// blocks in this CTA, in block order.  Returns false in the lanes without a
+// unit to finish here: past the batch, or split over CTAs whose others are
+// still to come (the last one takes the whole sum).  Called by all 32 lanes.
+__device__ __forceinline__ bool batch_sums(const StepParams &p, const BlockShared &sh, int32_t batch, int32_t &u,
+                                           double &s, int lane)
 {
-    uint32_t base = 0;
-    if (lane == 0 && n > 0)
-        base = atomicAdd(&pool.count, static_cast<uint32_t>(n));
-    base = __shfl_sync(kFull, base, 0);
-    if (lane < n) {
-        pool.unit[base + lane] = b;
-        pool.sumsq[base + lane] = s;
+    const int32_t i = batch * kBatch + lane, units = sh.cta.units;
+    u = sh.cta.unit + i;
+    bool active = i < units;
+    const int32_t lo = active && i > 0 ? sh.unit_end[i - 1] : 0, hi = active ? sh.unit_end[i] : 0;
+    // few units of many blocks: the warp sums each together
+    const bool wide = hi - lo > 8 && (units <= 4 || hi - lo > 64);
+    s = 0.0;
+    if (!wide)
+        for (int32_t j = lo; j < hi; ++j)
+            s += sh.sum[j];
+    for (unsigned m = __ballot_sync(kFull, wide); m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        const int32_t j0 = __shfl_sync(kFull, lo, l), j1 = __shfl_sync(kFull, hi, l);
+        double acc = 0.0;
+        for (int32_t j = j0 + lane; j < j1; j += 32)
+            acc += sh.sum[j];
+        acc = warp_allreduce_sum(acc);
+        if (lane == l)
+            s = acc;
     }
-    __threadfence_block();
-    __syncwarp();
-    uint32_t full = kNoBatch;
-    if (lane == 0) {
-        const uint32_t m = static_cast<uint32_t>(n), first = base / 32, room = 32 - base % 32;
-        const uint32_t m0 = m < room ? m : room;                       // units that went to batch `first`
-        uint32_t full2 = kNoBatch;                                     // later units may be there before earlier ones
-        if (m0 > 0 && atomicAdd(&pool.fill[first], m0) + m0 == 32)
-            full = first;
-        if (m > m0 && atomicAdd(&pool.fill[first + 1], m - m0) + m - m0 == 32)
-            full2 = first + 1;
-        __threadfence_block();
-        const bool last = atomicAdd(&pool.warps, 1u) + 1 == static_cast<uint32_t>(here);
-        if (full2 != kNoBatch)
-            pool.rest[atomicAdd(&pool.num_rest, 1u)] = full2;
-        if (last && full != kNoBatch) {
-            pool.rest[atomicAdd(&pool.num_rest, 1u)] = full;
-            full = kNoBatch;
+    // the units that may be split: both ends' exchanges travel together
+    const int e = i == 0 ? 0 : 1;
+    if (active && (i == 0 || i == units - 1) && sh.cta.parts[e] == 2)
+        active = exchange_parts(p, sh.cta.base[e], s);
+    for (int e = 0; e < 2; ++e) {
+        const int32_t at = e == 0 ? 0 : units - 1;
+        if (sh.cta.parts[e] <= 2 || at / kBatch != batch || (e == 1 && units == 1))
+            continue;
+        const int l = at % kBatch;
+        double x = __shfl_sync(kFull, s, l);
+        const bool whole = combine_parts(p, sh.cta.unit + at, sh.cta.parts[e], sh.cta.base[e], sh.cta.slot[e], x, lane);
+        if (lane == l) {
+            s = x;
+            active = whole;
         }
     }
-    full = __shfl_sync(kFull, full, 0);
-    __threadfence_block();
-    n = full != kNoBatch ? 32 : 0;
-    if (n) {
-        b = pool.unit[full * 32 + lane];
-        s = pool.sumsq[full * 32 + lane];
-    }
-}
-
-// After a barrier behind every warp's pool_leave(): the batch of this warp.
-// Returns its size.
-__device__ __forceinline__ int pool_rest(const EpiloguePool &pool, int32_t &b, double &s, int lane)
-{
-    const uint32_t wid = threadIdx.x >> 5, num_rest = pool.num_rest;
-    const int n = wid < num_rest ? 32 : wid == num_rest ? static_cast<int>(pool.count % 32) : 0;
-    if (lane < n) {
-        const uint32_t slot = (wid < num_rest ? pool.rest[wid] : pool.count / 32) * 32 + lane;
-        b = pool.unit[slot];
-        s = pool.sumsq[slot];
-    }
-    return n;
+    return active;
 }
 
 // MODE kStepFull: the whole step.  kStepPartials: phase 1 only, each unit's
@@ -981,17 +1101,38 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
 {
     __shared__ __align__(16) uint32_t s_hist[256];
     __shared__ uint32_t s_misc[8];
+    __shared__ int64_t s_t;
     __shared__ double s_red[kThreads];
-    extern __shared__ __align__(16) unsigned char s_keys[];   // kKeyCacheBytes unless MODE == kStepPartials
+    extern __shared__ __align__(16) unsigned char s_keys[];   // see launch_mode
     constexpr int kEB = Elem<DT>::kBytes;
     const int lane = threadIdx.x & 31;
     const int warp = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-    EpiloguePool &pool = *reinterpret_cast<EpiloguePool *>(s_keys);   // until the selection, which reuses it
-    if (MODE == kStepFull && Shape<V>::kPool && p.pool) {
-        if (threadIdx.x < kWarpsPerCta)
-            pool.fill[threadIdx.x] = 0;
-        if (threadIdx.x == kWarpsPerCta)
-            pool.count = pool.warps = pool.num_rest = 0;
+    BlockShared &sh = *reinterpret_cast<BlockShared *>(s_keys);
+    int32_t first_block = 0, blocks = 0;
+    Block cur{};
+    if (MODE != kStepFinish && Shape<V>::kBlocks) {
+        // The plan never changes after create: read while the kernel before
+        // this one on the stream is still running.
+        const CtaBlocks &plan = p.cta_blocks[blockIdx.x];
+        first_block = plan.first;
+        blocks = plan.count;
+        const int32_t unit = plan.unit, units = plan.units;
+        for (int32_t k = threadIdx.x; k < units; k += kThreads) {
+            const int32_t end = p.unit_block[unit + k + 1] - first_block;
+            sh.unit_end[k] = end < blocks ? end : blocks;
+        }
+        for (int32_t k = threadIdx.x; k * kBatch < units; k += kThreads) {
+            const int32_t u0 = unit + k * kBatch, n = units - k * kBatch;
+            const int32_t b0 = p.unit_block[u0] - first_block, b1 = p.unit_block[u0 + (n < kBatch ? n : kBatch)] - first_block;
+            sh.left[k] = (b1 < blocks ? b1 : blocks) - (b0 > 0 ? b0 : 0);
+        }
+        if (threadIdx.x == 0) {
+            sh.next = kWarpsPerCta;
+            sh.cta = plan;
+        }
+        const int32_t i = threadIdx.x >> 5;
+        if (i < blocks)
+            cur = p.block[first_block + i];
         __syncthreads();
     }
     // Launched as a programmatic dependent of whatever precedes it on the
@@ -1012,6 +1153,75 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             const double s = active ? p.in_sumsq[b] : 0.0;
             unit_epilogue(p, active, active ? static_cast<int32_t>(b) : 0, s, alpha, beta, t);
         }
+    } else if (Shape<V>::kBlocks) {
+        // t, alpha_t and beta_t are fixed for the whole step.
+        const int64_t t = MODE == kStepFull ? __ldcg(&p.ctl->steps) + 1 : 0;
+        const double alpha = pick_threshold(p.alpha_override, t, p.warmup_steps, p.alpha_init, p.alpha_main);
+        const double beta = pick_threshold(p.beta_override, t, p.warmup_steps, p.beta_init, p.beta_main);
+        const char *arena = static_cast<const char *>(p.arena);
+        // The state of the CTA's last batch of units, whose epilogue nothing hides.
+        if (MODE == kStepFull && threadIdx.x < kBatch && static_cast<int32_t>(threadIdx.x) < sh.cta.units) {
+            const int32_t u = sh.cta.unit + sh.cta.units - 1 - static_cast<int32_t>(threadIdx.x);
+            const double *Q = p.queue + static_cast<int64_t>(u) * p.window;
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(p.state + u));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(p.recoverable + u));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + p.window - 1));
+        }
+        // A warp that completes a batch runs it only when it has no block in
+        // hand: a block kept waiting for an epilogue would hold up its own batch.
+        int32_t i = threadIdx.x >> 5, batch = -1;
+        while (i < blocks) {
+            // the next block's index and table entry travel under this one's stream
+            int32_t next = blocks;
+            if (batch < 0) {
+                if (lane == 0)
+                    next = atomicAdd(&sh.next, 1);
+                next = __shfl_sync(kFull, next, 0);
+            }
+            const Block follow = p.block[first_block + (next < blocks ? next : i)];
+            const char *seg = arena + cur.start * kEB;
+            bool suspect;
+            double s = warp_segment_sumsq<DT, Shape<V>::kUnroll>(seg, cur.elems, lane, suspect);
+            if (suspect)
+                s = warp_segment_sumsq_f64<DT>(seg, cur.elems, lane);
+            int32_t left = 0;
+            if (lane == 0) {
+                sh.sum[i] = s;
+                __threadfence_block();
+                left = atomicSub(&sh.left[cur.batch], 1);
+            }
+            int32_t done = __shfl_sync(kFull, left, 0) == 1 ? cur.batch : -1;      // its last block
+            if (next >= blocks) {
+                __threadfence_block();
+                if (batch < 0) {
+                    batch = done;
+                    done = -1;
+                }
+                while (batch >= 0) {
+                    int32_t u;
+                    double sumsq;
+                    const bool active = batch_sums(p, sh, batch, u, sumsq, lane);
+                    if (MODE == kStepPartials) {
+                        if (active)
+                            p.out_sumsq[u] = sumsq;
+                    } else {
+                        unit_epilogue(p, active, u, sumsq, alpha, beta, t);
+                    }
+                    batch = done;
+                    done = -1;
+                }
+                if (lane == 0)
+                    next = atomicAdd(&sh.next, 1);
+                next = __shfl_sync(kFull, next, 0);
+                if (next < blocks)
+                    cur = p.block[first_block + next];
+            } else {
+                batch = done;
+                cur = follow;
+            }
+            i = next;
+        }
     } else if (warp < p.num_warps) {
         // t, alpha_t and beta_t are fixed for the whole step.
         const int64_t t = __ldcg(&p.ctl->steps) + 1;
@@ -1026,7 +1236,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         int32_t run = warp;                              // every warp starts on its own run
         auto complete = [&](int32_t b, double s) {
             const int32_t parts = p.num_parts[b];
-            if (parts == 1 || combine_parts(p, b, parts, run, s, lane)) {
+            if (parts == 1 || combine_parts(p, b, parts, p.part_base[b], run - p.first_run[b], s, lane)) {
                 if (MODE == kStepPartials) {
                     if (lane == 0)
                         p.out_sumsq[b] = s;
@@ -1036,17 +1246,17 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
                         pend_s = s;
                     }
                     if (++npend == 32) {
-                        unit_epilogue(p, true, pend_b, pend_s, alpha, beta, t);
+                        unit_epilogue_call(p, true, pend_b, pend_s, alpha, beta, t);
                         npend = 0;
                     }
                 }
             }
         };
         for (;;) {
-            // Large-unit loop: the index of the warp's next run is taken now, so
-            // the atomic's round trip hides under this run's stream.
+            // The index of the warp's next run is taken now, so the atomic's
+            // round trip hides under this run's stream.
             uint32_t next = 0;
-            if (Shape<V>::kDynamic && lane == 0)
+            if (lane == 0)
                 next = atomicAdd(&p.ctl->next_run, 1u);
             int64_t g = p.run_seg[run];
             int64_t pos = p.run_pos[run];
@@ -1080,8 +1290,6 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             }
             if (cur >= 0)
                 complete(cur, cur_s);
-            if (!Shape<V>::kDynamic)
-                break;
             run = p.num_warps + static_cast<int32_t>(__shfl_sync(kFull, next, 0));
             if (run >= p.num_runs)
                 break;
@@ -1090,53 +1298,39 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         // after this grid has completed) by the selecting CTA, after every
         // warp has drawn its last index.  The partial-sums half has no
         // selecting CTA: there the last warp to draw past the end resets it.
-        if (Shape<V>::kDynamic && MODE == kStepPartials && lane == 0 &&
+        if (MODE == kStepPartials && lane == 0 &&
             ticket_acq_rel(&p.ctl->warps_done) == static_cast<uint32_t>(p.num_warps - 1)) {
             p.ctl->next_run = 0;
             p.ctl->warps_done = 0;
         }
         if (MODE == kStepFull) {
-            if (Shape<V>::kPool && p.pool) {
-                const int32_t here = p.num_warps - static_cast<int32_t>(blockIdx.x) * kWarpsPerCta;   // with a first run
-                pool_leave(pool, here < kWarpsPerCta ? here : kWarpsPerCta, npend, pend_b, pend_s, lane);
-            }
             if (npend > 0)
-                unit_epilogue(p, lane < npend, pend_b, pend_s, alpha, beta, t);
+                unit_epilogue_call(p, lane < npend, pend_b, pend_s, alpha, beta, t);
         }
     }
     if (MODE == kStepPartials)
         return;
 
-    if (MODE == kStepFull && Shape<V>::kPool && p.pool) {
-        __syncthreads();
-        int32_t b = 0;
-        double sumsq = 0.0;
-        const int n = pool_rest(pool, b, sumsq, lane);
-        if (n > 0) {
-            const int64_t t = __ldcg(&p.ctl->steps) + 1;
-            unit_epilogue(p, lane < n, b, sumsq,
-                          pick_threshold(p.alpha_override, t, p.warmup_steps, p.alpha_init, p.alpha_main),
-                          pick_threshold(p.beta_override, t, p.warmup_steps, p.beta_init, p.beta_main), t);
-        }
-    }
-
     // Grid completion: the last CTA through runs the selection.  The barrier
     // orders the CTA's writes before thread 0's release; the last ticket's
     // acquire, then the barrier, orders the selecting CTA's reads after
     // every CTA's writes.
+    if (threadIdx.x == 0)
+        s_t = __ldcg(&p.ctl->steps) + 1;
     __syncthreads();
     if (threadIdx.x == 0)
         s_misc[kMiscLast] = ticket_acq_rel(&p.ctl->ctas_done) == gridDim.x - 1 ? 1u : 0u;
     __syncthreads();
     if (s_misc[kMiscLast]) {
-        select_and_commit(p, __ldcg(&p.ctl->steps) + 1, s_hist, s_misc, s_red, s_keys);
+        select_and_commit(p, s_t, s_hist, s_misc, s_red, s_keys);
     }
 }
 
 template <int MODE, int V>
 cudaError_t launch_mode(const StepParams &p, int dtype, int num_ctas, cudaStream_t stream)
 {
-    constexpr size_t smem = MODE == kStepPartials ? 0 : kKeyCacheBytes;
+    constexpr size_t smem = MODE != kStepPartials ? kKeyCacheBytes : Shape<V>::kBlocks ? sizeof(BlockShared) : 0;
+    static_assert(sizeof(BlockShared) <= kKeyCacheBytes && sizeof(BlockShared) <= (48u << 10), "block sums' shared memory");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(num_ctas));
     cfg.blockDim = dim3(kThreads);

@@ -130,4 +130,79 @@ bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int3
     return true;
 }
 
+// Blocks: the pieces of one segment that a CTA's warps take in turn.  The sums
+// of a CTA's blocks live in its shared memory, kBlocksPerCta of them at most:
+// larger blocks first, then more CTAs than are resident, make room.
+bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t *seg_lengths,
+                 const int32_t *seg_unit, int32_t num_units, int elem_bytes, int32_t max_ctas, Plan &out,
+                 BlockPlan &blocks)
+{
+    if (num_segments < 1 || !seg_offsets || !seg_lengths || !seg_unit || max_ctas < 1)
+        return false;
+    int64_t cost = int64_t(num_units) * kUnitCostBytes;
+    for (int64_t g = 0; g < num_segments; ++g) {
+        if (seg_lengths[g] < 0 || seg_lengths[g] > (INT64_MAX / 8) / elem_bytes ||
+            cost > INT64_MAX / 2 - seg_lengths[g] * elem_bytes)
+            return false;
+        cost += seg_lengths[g] * elem_bytes;
+    }
+    int64_t ctas = std::min<int64_t>(max_ctas, std::max<int64_t>(1, cost / kMinCtaBytes));
+    const int64_t granule = kSplitBytes / elem_bytes;
+    for (int64_t bytes = kMinBlockBytes;;) {
+        if (ctas > INT32_MAX / 2 || !plan_partition(num_segments, seg_lengths, seg_unit, num_units, elem_bytes,
+                                                    static_cast<int32_t>(ctas), out))
+            return false;
+        blocks.cta.clear();
+        blocks.block.clear();
+        blocks.unit_block.assign(num_units + 1, 0);
+        bool fits = true;
+        int32_t prev_unit = -1;
+        for (int32_t r = 0; r < out.num_runs && fits; ++r) {
+            CtaBlocks c{};
+            c.first = static_cast<int32_t>(blocks.block.size());
+            c.unit = seg_unit[out.run_seg[r]];
+            int64_t pos = out.run_pos[r];
+            for (int64_t g = out.run_seg[r]; g < out.run_seg[r + 1] || (g == out.run_seg[r + 1] && pos < out.run_pos[r + 1]);
+                 ++g, pos = 0) {
+                const int64_t stop = g == out.run_seg[r + 1] ? std::min(out.run_pos[r + 1], seg_lengths[g]) : seg_lengths[g];
+                const int64_t n = std::max<int64_t>(stop - pos, 0);
+                const int32_t u = seg_unit[g];
+                if (u != prev_unit)
+                    blocks.unit_block[u] = static_cast<int32_t>(blocks.block.size());
+                prev_unit = u;
+                // equal pieces of whole granules; an empty segment is one empty piece
+                const int64_t pieces = std::max<int64_t>(1, (n * elem_bytes + bytes - 1) / bytes);
+                const int64_t per = ((n + pieces - 1) / pieces + granule - 1) / granule * granule;
+                int64_t at = 0;
+                do {
+                    const int64_t m = std::min(std::max<int64_t>(per, 1), n - at);
+                    blocks.block.push_back({seg_offsets[g] + pos + at, static_cast<int32_t>(m), (u - c.unit) / kBatch});
+                    at += m;
+                } while (at < n);
+                c.units = u - c.unit + 1;
+                if (blocks.block.size() - c.first > size_t(kBlocksPerCta) || blocks.block.size() > size_t(INT32_MAX / 2)) {
+                    fits = false;
+                    break;
+                }
+            }
+            c.count = static_cast<int32_t>(blocks.block.size()) - c.first;
+            for (int e = 0; e < 2; ++e) {
+                const int32_t u = e == 0 ? c.unit : c.unit + c.units - 1;
+                c.parts[e] = out.num_parts[u];
+                c.slot[e] = r - out.first_run[u];
+                c.base[e] = out.part_base[u];
+            }
+            blocks.cta.push_back(c);
+        }
+        if (fits) {
+            blocks.unit_block[num_units] = static_cast<int32_t>(blocks.block.size());
+            return true;
+        }
+        if (bytes < kMaxBlockBytes)
+            bytes *= 2;
+        else
+            ctas *= 2;
+    }
+}
+
 }  // namespace gnmr

@@ -2,8 +2,8 @@
 // ticket, shared by the step kernel and the allocation-free norms entry point
 // (device code only).
 //
-// A warp reads a segment with 16-byte loads on the non-coherent path (no L1
-// allocation, 256-byte L2 prefetch), squares in fp32, sums short blocks in
+// A warp reads a segment with 16-byte loads (no L1 allocation, 256-byte L2
+// prefetch), squares in fp32, sums short blocks in
 // fp32 and the blocks as an unevaluated pair of floats (hi + lo, about 48
 // significant bits), then adds the 32 lanes' totals with an fp32 xor
 // butterfly (non-negative terms: at most five roundings, about 3e-7
@@ -41,8 +41,10 @@ template <> struct Elem<1> {             // bf16, two per 32-bit word
     static constexpr uint32_t kMagnitude = 0x7fff7fffu;
 };
 
-// 16-byte streaming load: non-coherent read-only path, no L1 allocation,
-// 256-byte L2 prefetch granularity.
+// 16-byte streaming load: no L1 allocation, 256-byte L2 prefetch granularity.
+// A coherent load, and volatile like the element loads below: a kernel that
+// was started early (griddepcontrol) knows its addresses before the data is
+// written, so no load may move up over the wait.
 constexpr int kVecWords = 4;
 constexpr int kVecBytes = 16;
 struct alignas(kVecBytes) Vec {
@@ -52,7 +54,7 @@ struct alignas(kVecBytes) Vec {
 __device__ __forceinline__ Vec ld_stream(const Vec *p)
 {
     Vec r;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
         : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]) : "l"(p));
     return r;
 }
@@ -79,11 +81,15 @@ __device__ __forceinline__ uint32_t vec_or(const Vec &v)
 template <int DT> __device__ __forceinline__ uint32_t ld_elem_bits(const char *p);
 template <> __device__ __forceinline__ uint32_t ld_elem_bits<0>(const char *p)
 {
-    return __ldg(reinterpret_cast<const unsigned int *>(p));
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
 }
 template <> __device__ __forceinline__ uint32_t ld_elem_bits<1>(const char *p)
 {
-    return static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short *>(p))) << 16;
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return static_cast<uint32_t>(v) << 16;
 }
 
 // Sum of squares of the elements packed in one vector, in fp32 (two

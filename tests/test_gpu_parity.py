@@ -717,12 +717,12 @@ def test_steps_wait_for_the_kernel_that_writes_the_arena(config, shrink, cuda_de
         mon.close()
 
 
-@pytest.mark.parametrize("units_per_sm,extra", [(6, -1), (6, 0), (6, 1), (13, 0), (32, 1), (133, 3), (520, 0)])
-def test_pooled_epilogues_update_every_unit_once(units_per_sm, extra, cuda_device):
-    """Layouts of 6 units per SM up to 16 per warp run their last epilogue
-    batches from a pool of the CTA's units.  The controller half runs them
-    unit by unit, so both must leave the same state, masks and statistics,
-    bit for bit, on the same sums."""
+@pytest.mark.parametrize("units_per_sm,extra", [(1, 0), (6, 1), (13, 0), (32, 1), (133, 3), (520, 0)])
+def test_small_unit_batches_update_every_unit_once(units_per_sm, extra, cuda_device):
+    """The small-unit loop runs the epilogues in batches of 32 units of a CTA,
+    by whichever warp completes one.  The controller half runs them unit by
+    unit, so both must leave the same state, masks and statistics, bit for
+    bit, on the same sums."""
     import torch
     U = units_per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
     rng = np.random.default_rng(U)
@@ -744,3 +744,37 @@ def test_pooled_epilogues_update_every_unit_once(units_per_sm, extra, cuda_devic
     finally:
         one.close()
         two.close()
+
+
+def _block_layout(name):
+    if name == "block-edges":                             # around one and two blocks of 8 KiB
+        return np.repeat([0, 1, 2047, 2048, 2049, 4095, 4096, 4097, 6145], 40)
+    if name == "cta-spans":                               # units over two, three and more CTAs' parts
+        return np.array([5_000, 30_001, 12_000, 20_000, 7, 90_003, 1, 0, 50_000, 64_001])
+    if name == "more-than-resident":                      # more units than the resident CTAs' blocks
+        return np.arange(700_001) % 4
+    return np.array([70_000_001, 3, 0, 12_345])           # "one-giant": blocks larger than 8 KiB
+
+
+@pytest.mark.parametrize("name", ["block-edges", "cta-spans", "more-than-resident", "one-giant"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_block_loop_layouts(name, dtype, cuda_device):
+    """Norms of the small-unit loop at the edges of its plan, at odd offsets,
+    against 64-bit sums, twice (the second step reuses every slot)."""
+    import torch
+    lengths = _block_layout(name).astype(np.int64)
+    offsets = np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64) + 1
+    n = int(lengths.sum()) + 1
+    ids = torch.repeat_interleave(torch.arange(len(lengths), device=cuda_device),
+                                  torch.from_numpy(lengths).to(cuda_device))
+    with Monitor(offsets, lengths, dtype=dtype, loop_shape="small", window=2) as mon:
+        stats = mon.new_stats()
+        for seed in (1, 2):
+            g = torch.Generator(cuda_device).manual_seed(seed)
+            arena = torch.randn(n, device=cuda_device, generator=g).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+            mon.step(arena, stats=stats)
+            want = torch.zeros(len(lengths), dtype=torch.float64, device=cuda_device)
+            want.index_add_(0, ids, arena[1:].double().square())
+            # a piece's fp32 sum: at most about 27 roundings of 2^-24 per block
+            # of 16 iterations and 5 over the lanes, halved by the square root
+            torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=1e-6, atol=0)
