@@ -97,10 +97,8 @@ constexpr uint32_t kCandActive = 0x80000000u;
 
 // Risk histogram of the candidate pool, built by the unit epilogues with one
 // atomic per pool member and read (and cleared) by the selecting CTA.  Bin 0
-// holds R < 1 (lock-only candidates); bin i >= 1 holds the R >= 1 whose
-// exponent and top three mantissa bits are the (i-1)-th such pattern above
-// 1.0: eight bins per octave, [1, 1.125), [1.125, 1.25), ..., [1.875, 2),
-// [2, 2.25), ...; the last bin also holds everything larger (+inf included).
+// holds R < 1 (lock-only candidates); the bins above 1.0 get wider with R
+// (risk_bin); the last one also holds everything larger (+inf included).
 constexpr int kRiskBins = 2048;
 // Hot list: the candidates a step appends because their bin is at or above a
 // bin predicted from the previous step's cut (plus, under the admission cap,

@@ -106,39 +106,65 @@ __device__ __forceinline__ uint32_t index_key(int32_t b, int32_t num_units)
 }
 
 // Bin of the risk histogram for a risk key (non-decreasing in the key): 0 for
-// R < 1, else 1 + the key's exponent and top three mantissa bits counted
-// from those of 1.0, the last bin open-ended.
+// R < 1, then kFineBins of 128 per octave up to 2^8, kMidBins of 32 per octave
+// up to 2^24, and 8 per octave from there, the last bin open-ended.  The cut
+// falls among moderate risks, where the bins are narrow, so that few members of
+// its bin are left to rank: with 8 per octave throughout, cuts at R of 4 to 6
+// left 440-660 members (1,400 candidates) to 2,455 (4,900), now 85-122 to 489.
+constexpr int kFineOctaves = 8, kFineBits = 7, kFineBins = kFineOctaves << kFineBits;
+constexpr int kMidOctaves = 16, kMidBits = 5, kMidBins = kMidOctaves << kMidBits;
+constexpr int kCoarseBits = 3;
+static_assert(1 + kFineBins + kMidBins < kRiskBins, "room for the coarse bins");
 __device__ __forceinline__ uint32_t risk_bin(uint64_t key)
 {
-    constexpr uint32_t kOne = 1023u << 3;                 // exponent of 1.0, three mantissa bits 0
-    const uint32_t e8 = static_cast<uint32_t>(key >> 49); // sign (0), exponent, top three mantissa bits
-    if (e8 < kOne)
+    constexpr uint32_t kOne = 1023;                                  // exponent of 1.0
+    const uint32_t e = static_cast<uint32_t>(key >> 52);             // sign (0) and exponent
+    if (e < kOne)
         return 0;
-    const uint32_t b = e8 - kOne + 1;
+    if (e < kOne + kFineOctaves)
+        return 1 + static_cast<uint32_t>(key >> (52 - kFineBits)) - (kOne << kFineBits);
+    if (e < kOne + kFineOctaves + kMidOctaves)
+        return 1 + kFineBins + static_cast<uint32_t>(key >> (52 - kMidBits)) - ((kOne + kFineOctaves) << kMidBits);
+    const uint32_t b = 1 + kFineBins + kMidBins + static_cast<uint32_t>(key >> (52 - kCoarseBits)) -
+                       ((kOne + kFineOctaves + kMidOctaves) << kCoarseBits);
     return b < static_cast<uint32_t>(kRiskBins) ? b : static_cast<uint32_t>(kRiskBins - 1);
 }
 
-// Appends the lanes' entries (flag set) to a list with one atomic per warp;
-// slots at or past cap are counted but not written.  Called by all 32 lanes.
-__device__ __forceinline__ void warp_append(Candidate *list, uint32_t *count, uint32_t cap, bool flag, double r,
-                                            int32_t b, uint32_t lk)
+// Lowest key bit above which all keys of bin c agree (64: none have to).
+__device__ __forceinline__ int bin_shared_bit(uint32_t c)
 {
-    const unsigned want = __ballot_sync(kFull, flag);
+    if (c == 0 || c + 1 >= static_cast<uint32_t>(kRiskBins))
+        return 64;
+    return 52 - (c <= kFineBins ? kFineBits : c <= kFineBins + kMidBins ? kMidBits : kCoarseBits);
+}
+
+// Appends the lanes' entries to the candidate list (cand) and to the hot list
+// (hot) with one atomic per warp and list, both in flight together; slots at or
+// past a list's end are counted but not written.  Called by all 32 lanes.
+__device__ __forceinline__ void append_candidates(const StepParams &p, bool cand, bool hot, double r, int32_t b,
+                                                  uint32_t lk)
+{
+    const unsigned want = __ballot_sync(kFull, cand), want_hot = __ballot_sync(kFull, hot);
     if (!want)
-        return;
+        return;                                          // hot entries are candidates
     const int lane = threadIdx.x & 31;
-    const int leader = __ffs(want) - 1;
     uint32_t base = 0;
-    if (lane == leader)
-        base = atomicAdd(count, static_cast<uint32_t>(__popc(want)));
-    base = __shfl_sync(kFull, base, leader);
-    if (flag) {
-        const uint32_t slot = base + __popc(want & ((1u << lane) - 1u));
-        if (slot < cap) {
-            list[slot].risk = r;
-            list[slot].unit = b;
-            list[slot].lock = lk;
-        }
+    if (lane == 0)
+        base = atomicAdd(&p.ctl->n_cand, static_cast<uint32_t>(__popc(want)));
+    else if (lane == 1 && want_hot)
+        base = atomicAdd(&p.ctl->n_hot, static_cast<uint32_t>(__popc(want_hot)));
+    const uint32_t below = (1u << lane) - 1u;
+    const uint32_t slot = __shfl_sync(kFull, base, 0) + __popc(want & below);
+    const uint32_t slot_hot = __shfl_sync(kFull, base, 1) + __popc(want_hot & below);
+    if (cand && slot < static_cast<uint32_t>(p.num_units)) {
+        p.cand[slot].risk = r;
+        p.cand[slot].unit = b;
+        p.cand[slot].lock = lk;
+    }
+    if (hot && slot_hot < p.hot_cap) {
+        p.hot[slot_hot].risk = r;
+        p.hot[slot_hot].unit = b;
+        p.hot[slot_hot].lock = lk;
     }
 }
 
@@ -335,8 +361,7 @@ __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, doubl
         atomicAdd(&p.risk_hist[bin], 1u);
         hot = bin >= hot_bin;
     }
-    warp_append(p.cand, &p.ctl->n_cand, static_cast<uint32_t>(p.num_units), cand, r, b, cand_lock);
-    warp_append(p.hot, &p.ctl->n_hot, p.hot_cap, hot, r, b, cand_lock);
+    append_candidates(p, cand, hot, r, b, cand_lock);
 }
 
 // The same, out of line: the large-unit loop calls it rarely and keeps its
@@ -621,18 +646,22 @@ __device__ __forceinline__ void find_bucket_wide(const uint32_t *hist, uint32_t 
     }
 }
 
-// Reads and clears the global risk histogram (four bins per thread, thread 0
-// the highest).  misc[kMiscPool] = the pool size P; with K = min(P, cap),
+// The thread's four bins of the global risk histogram, thread 0 the highest.
+__device__ __forceinline__ uint4 *own_bins(const StepParams &p)
+{
+    return reinterpret_cast<uint4 *>(p.risk_hist) + (kRiskBins / 4 - 1 - static_cast<int>(threadIdx.x));
+}
+
+// Clears the global risk histogram and scans what it held (q: own_bins()).  misc[kMiscPool] = the pool size P; with K = min(P, cap),
 // if 1 <= K < P: misc[kMiscBin/Rank/Count] describe the bin holding the K-th
 // largest risk, and misc[kMiscHint] the bin holding the min(P, K + extra)-th
 // largest (the next step's hot-list prediction).  Callers synchronise after.
-__device__ void scan_risk_hist(const StepParams &p, uint32_t cap, uint32_t extra, uint32_t *misc, uint32_t *wsum)
+__device__ void scan_risk_hist(const StepParams &p, const uint4 q, uint32_t cap, uint32_t extra, uint32_t *misc,
+                               uint32_t *wsum)
 {
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const int q4 = kRiskBins / 4 - 1 - t;
-    uint4 *gh = reinterpret_cast<uint4 *>(p.risk_hist) + q4;
-    const uint4 q = __ldcg(gh);                                      // bins 4 q4 .. 4 q4 + 3
-    __stcg(gh, make_uint4(0u, 0u, 0u, 0u));                          // empty for the next step
+    __stcg(own_bins(p), make_uint4(0u, 0u, 0u, 0u));                 // empty for the next step
     const uint32_t c4[4] = {q.w, q.z, q.y, q.x};                     // descending
     const uint32_t sum = c4[0] + c4[1] + c4[2] + c4[3];
     uint32_t incl = sum;
@@ -800,10 +829,14 @@ __device__ __forceinline__ uint32_t ranks_above(uint64_t kj, int32_t uj, uint64_
 }
 
 // Commits the r largest (key desc, unit asc) of the n cut-list entries,
-// 1 <= r < n <= kCutCap.  Each entry's rank is counted against all others
-// directly: up to 32 entries in warp 0's registers (shuffles), up to one per
-// thread from shared memory (eight entries per step, loads issued together);
-// larger lists use the radix select.
+// 1 <= r < n <= kCutCap.  Small lists: each entry's rank is counted against all
+// others directly, up to 32 entries in warp 0's registers (shuffles), up to
+// kRankMax one per thread from shared memory (eight entries per step, loads
+// issued together); larger lists use the radix select (one or two passes of
+// about 0.7 us).  The direct count grows with n^2: with 512 in place of 128 the
+// 100K-unit step took 244.5 us instead of 240.4.
+constexpr uint32_t kRankMax = 128;
+static_assert(kRankMax <= kThreads, "one entry per thread");
 __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t n, uint32_t r, const uint64_t *ck,
                            const int32_t *cu, const uint32_t *cl, uint32_t *hist, uint32_t *wsum, uint32_t *misc)
 {
@@ -825,7 +858,7 @@ __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t 
         }
         return;
     }
-    if (n <= blockDim.x) {
+    if (n <= kRankMax) {
         const uint32_t i = threadIdx.x;
         if (i < n) {
             const uint64_t k = ck[i];
@@ -851,8 +884,7 @@ __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t 
         }
         return;
     }
-    // every key of an interior bin shares the sign, exponent and top three mantissa bits
-    const int start = (c > 0 && c + 1 < static_cast<uint32_t>(kRiskBins)) ? 49 : 64;
+    const int start = bin_shared_bit(c);
     uint64_t thr_hi = 0;
     uint32_t thr_lo = 0;
     radix_select_cut(ck, cu, n, r, start, p.num_units, hist, wsum, misc, thr_hi, thr_lo);
@@ -880,9 +912,14 @@ __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t 
 __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist, uint32_t *misc, double *red,
                                   unsigned char *smem)
 {
-    uint32_t m = 0;
+    // one round trip for all that the selection starts from
+    uint32_t m = 0, n_hot = 0, hot_bin = 0;
+    uint4 bins = make_uint4(0u, 0u, 0u, 0u);
     if (!p.dense) {
         m = __ldcg(&p.ctl->n_cand);
+        n_hot = __ldcg(&p.ctl->n_hot);
+        hot_bin = __ldcg(&p.ctl->hot_bin);
+        bins = __ldcg(own_bins(p));
         m = m < static_cast<uint32_t>(p.num_units) ? m : static_cast<uint32_t>(p.num_units);
     }
     const bool all_on = t <= p.forced_steps || (p.policy == 2 && t <= p.static_warmup);
@@ -957,7 +994,7 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
         next_hot = 0;                                // a small pool: every candidate is hot next step
     } else {
         const uint32_t cap = stat ? static_cast<uint32_t>(p.static_keep) : static_cast<uint32_t>(p.max_o);
-        scan_risk_hist(p, cap, 3 * cap + 64, misc, hist);
+        scan_risk_hist(p, bins, cap, 3 * cap + 64, misc, hist);
         __syncthreads();
         const uint32_t pool = misc[kMiscPool];
         const uint32_t retained = admission && m > pool ? m - pool : 0u;
@@ -981,8 +1018,6 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
             uint32_t *wide_hist = reinterpret_cast<uint32_t *>(smem + kCutHistOffset);
             const uint32_t c = misc[kMiscBin], rc = misc[kMiscRank], nc = misc[kMiscCount];
             next_hot = misc[kMiscHint];
-            const uint32_t hot_bin = __ldcg(&p.ctl->hot_bin);
-            const uint32_t n_hot = __ldcg(&p.ctl->n_hot);
             const bool use_hot = hot_bin <= c && n_hot <= p.hot_cap;
             __syncthreads();                         // every thread has read misc
             if (threadIdx.x == 0)

@@ -9,10 +9,11 @@ correctly rounded fp64 operations, so R, the masks, the locks and the counts
 must agree exactly -- no decision margin is needed, and ties are real.
 
 The cases steer the selection through each of its paths.  The risk
-histogram (eight bins per octave: exponent and top three mantissa bits)
-locates the cut bin; its members are ranked directly (up to 512), by a radix
+histogram (128 bins per octave up to 2^8, 32 up to 2^24, 8 above) locates the
+cut bin; its members are ranked directly (up to 128), by a radix
 select in shared memory (up to 3,072), or by radix passes over the whole
 candidate list in global memory (more); a cut bin can also be taken whole.
+Up to 2,048 units there is no histogram: the whole pool is ranked that way.
 Multi-step cases drive the hot list: the previous step's prediction held
 (only the hot list is read), missed (the risks fell below it), or the hot
 list overflowed.  Equal risks inside the cut bin, lock-only candidates and
@@ -234,3 +235,50 @@ def test_random_small_controllers_agree_exactly(seed, cuda_device):
     finally:
         mon.close()
         ctl.close()
+
+
+# Members of one bin of each width, below 2^8, below 2^24 and above.
+BIN_OF = {"fine": (8.0, 8.06), "mid": (512.0, 527.9), "coarse": (2.0 ** 25, 2.0 ** 25 * 1.124)}
+
+
+@pytest.mark.parametrize("width", sorted(BIN_OF))
+@pytest.mark.parametrize("n_cut", [55, 128, 129, 3072, 3073])
+def test_cut_in_bins_of_each_width(width, n_cut, cuda_device):
+    rng = np.random.default_rng(n_cut)
+    r = rng.uniform(0.5, 0.9, U)
+    top = rng.choice(U, 10 + n_cut, replace=False)
+    lo, hi = BIN_OF[width]
+    r[top[:10]] = hi * 2.0 + np.arange(10)
+    r[top[10:]] = rng.uniform(lo, hi, n_cut)
+    assert _drive([r, r]).n_selected == min(MAX_O, 10 + n_cut)
+
+
+@pytest.mark.parametrize("edge", [1.0, 2.0 ** 8, 2.0 ** 24, 2.0 ** 87, 2.0 ** 88, 2.0 ** 200])
+def test_cut_across_a_change_of_bin_width(edge, cuda_device):
+    rng = np.random.default_rng(7)
+    r = rng.uniform(0.5, 0.9, U)
+    top = rng.choice(U, 400, replace=False)
+    r[top] = edge * np.exp2(rng.uniform(-0.02, 0.02, 400))
+    r[top[:50]] = edge
+    _drive([r, r])
+
+
+@pytest.mark.parametrize("units", [1, 33, 512, 513, 2047, 2048, 2049])
+@pytest.mark.parametrize("kind", ["spread", "ties", "fits", "none"])
+def test_selection_of_few_units(units, kind, cuda_device, monkeypatch):
+    """Around the 2,048 units up to which the selection reads every unit:
+    active cap over several steps (locks, retained locks), admission cap and
+    the static policy."""
+    monkeypatch.setitem(globals(), "U", units)
+    rng = np.random.default_rng(units)
+    def risks():
+        if kind == "none":
+            return rng.uniform(0.2, 0.9, units)
+        r = np.full(units, 3.0) if kind == "ties" else np.exp(rng.uniform(np.log(0.5), np.log(1e4), units))
+        if kind == "fits":
+            r[rng.permutation(units)[MAX_O // 2:]] = 0.5
+        return r
+    steps = [risks() for _ in range(4)]
+    _drive(steps)
+    _drive(steps, policy=1)
+    _drive(steps, policy=2, static_warmup_steps=2, static_fraction=0.3)
