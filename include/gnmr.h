@@ -360,8 +360,8 @@ gnmr_status gnmr_actuator_destroy(gnmr_actuator *a);
  *
  * Limit: num_units <= 131072 (any arena size); beyond it
  * GNMR_ERR_INVALID_ARG, with gnmr_last_error(NULL) reading "units > 131072".
- * The arena is read as 64 KiB chunks split into contiguous ranges over the
- * GPU's warps, at the step kernel's streaming rate.  A unit outside [0, arena_elems)
+ * The arena is read in contiguous ranges of about equal cost, one per warp of
+ * the GPU, at the step kernel's streaming rate.  A unit outside [0, arena_elems)
  * gives GNMR_ERR_LAYOUT ("unit off arena"); other details: "dtype unknown",
  * "NULL pointer", "arena misalign", "CUDA failed", "device query" (the
  * current device or its SM count could not be read).  The call makes no host
@@ -371,7 +371,8 @@ gnmr_status gnmr_actuator_destroy(gnmr_actuator *a);
  * device; make that first call before any stream capture.  The layout tables
  * are uploaded (pageable host->device copies) only when the layout, dtype or
  * device differs from the previous call's; a call repeating the previous
- * layout enqueues one memset and one kernel.  Every call shares the one
+ * layout enqueues one kernel, and one before it that clears the tickets if some
+ * unit is shared by several warps.  Every call shares the one
  * array and leaves its contents behind (each call clears what must start at
  * zero); calls that overlap on the GPU race on it, so callers must serialise
  * them (one stream, one thread at a time).  Each upload tags the tables with

@@ -36,7 +36,11 @@ using gnmr::kFull;
 
 constexpr int64_t kMaxUnits = int64_t(1) << 17;        // 131,072 units
 constexpr int64_t kMaxWarps = int64_t(1) << 14;        // streaming warps of one call
-constexpr int64_t kChunkBytes = int64_t(64) << 10;     // gradient bytes per chunk
+// Gradient bytes per chunk, the granularity at which warp ranges are cut: fine,
+// or so coarse that a layout of small units is not cut inside a unit at all
+// (then no ticket has to be cleared, which saves a launch).
+constexpr int kFineShift = 12, kCoarseShift = 14;      // log2: 4 KiB, 16 KiB
+constexpr int64_t kSpanBytes = int64_t(64) << 10;      // bytes of a unit summed in one go
 constexpr int kThreads = 512;
 constexpr int kWarpsPerCta = kThreads / 32;
 constexpr int kUnroll = 8;                             // 16-byte loads in flight per lane
@@ -89,6 +93,18 @@ __host__ __device__ inline View carve(unsigned char *base)
                 reinterpret_cast<double *>(base + kOffPartial)};
 }
 
+// Clears the units' tickets, in a launch of its own that the norms kernel can
+// start under; behind a memset node it cannot (64 units, graph-replayed: 7.8 us
+// against 11.3).
+__global__ void __launch_bounds__(kThreads) clear_tickets_kernel(uint32_t *ticket, int32_t num_units)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int32_t u = static_cast<int32_t>(blockIdx.x * blockDim.x + threadIdx.x); u < num_units;
+         u += static_cast<int32_t>(gridDim.x * blockDim.x))
+        ticket[u] = 0;
+}
+
 // Chunks of unit b: ceil(length / chunk_elems), at least one (an empty unit
 // still gets its norm, 0, written).  chunk_elems = 2^chunk_shift.
 __host__ __device__ inline int64_t unit_chunks(int64_t len, int chunk_shift)
@@ -106,9 +122,15 @@ __host__ __device__ inline int64_t unit_chunks(int64_t len, int chunk_shift)
 // unit is fixed.
 
 // Warp w streams its contiguous range of chunks with the step kernel's
-// segment reduction, adding the chunks of one unit in order; a unit held by
-// one warp is finished there, a unit spread over several by the warp that
-// takes its last ticket, which adds the pieces in slot order.
+// segment reduction, up to kSpanBytes of one unit at a time, adding them in
+// order; a unit held by one warp is finished there, a unit spread over several
+// by the warp that takes its last ticket, which adds the pieces in slot order.
+// Finished units wait in the warp's lanes for their square roots: an fp64 one
+// holds the SM's fp64 pipe for about 0.1 us whatever its active lanes.
+// HBM-bound.  With ranges cut at 64 KiB a warp had one chunk or two where the
+// mean was 1.6 (3,000 units, 509 MB: 91.5 -> 81.1 us on one GB300, with the
+// programmatic launches; 2,600 odd bf16 units 33.5 -> 17.0; 64 units 16.4 ->
+// 11.6; 100K units 239.5 -> 229.1; 280 units in 25 GB 3441 -> 3436).
 //
 // `generation` is the layout generation the call enqueued its work for.  If
 // the tables in the scratch array hold another one (a call with a different
@@ -117,12 +139,14 @@ __host__ __device__ inline int64_t unit_chunks(int64_t len, int chunk_shift)
 template <int DT>
 __global__ void __launch_bounds__(kThreads, 2) static_norms_kernel(const void *arena, unsigned char *base,
                                                                    int32_t num_units, int64_t W,
-                                                                   int64_t chunk_elems, double *norms,
+                                                                   int chunk_shift, double *norms,
                                                                    unsigned long long generation)
 {
     constexpr int kEB = gnmr::Elem<DT>::kBytes;
     const View v = carve(base);
     const int lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t w = static_cast<int64_t>(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
     if (__ldcg(v.generation) != generation) {
         const int64_t threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -171,6 +195,15 @@ __global__ void __launch_bounds__(kThreads, 2) static_norms_kernel(const void *a
     meta(b);
     double s = 0.0;
 
+    // Units this warp finishes, lane j holding the j-th.
+    int32_t pend_u = 0;
+    double pend_s = 0.0;
+    int npend = 0;
+    auto write_pending = [&]() {
+        if (lane < npend)
+            norms[pend_u] = sqrt(pend_s);
+        npend = 0;
+    };
     auto finish = [&](int32_t u, int64_t u_wp, double sum) {
         const int64_t w0 = static_cast<uint32_t>(u_wp);
         const int64_t pieces = u_wp >> 32;
@@ -191,16 +224,21 @@ __global__ void __launch_bounds__(kThreads, 2) static_norms_kernel(const void *a
             if (lane == 0)
                 v.ticket[u] = 0;                         // ready for the next call
         }
-        if (lane == 0)
-            norms[u] = sqrt(sum);
+        if (lane == npend) {
+            pend_u = u;
+            pend_s = sum;
+        }
+        if (++npend == 32)
+            write_pending();
     };
 
-    for (int64_t c = c0; c < c1; ++c) {
+    for (int64_t c = c0; c < c1;) {
         if (c >= next) {                                 // the range moves on to the next unit
             finish(b, wp, s);
             s = 0.0;
             do {
                 if (b + 1 >= num_units) {                // tables not of this layout: stop
+                    write_pending();
                     if (lane == 0)
                         norms[b] = CUDART_NAN;
                     return;
@@ -208,8 +246,12 @@ __global__ void __launch_bounds__(kThreads, 2) static_norms_kernel(const void *a
                 meta(++b);
             } while (c >= next);
         }
-        const int64_t a = (c - first) * chunk_elems;
-        const int64_t e = a + chunk_elems < len ? a + chunk_elems : len;
+        int64_t stop = c1 < next ? c1 : next;
+        const int64_t most = (kSpanBytes / kEB) >> chunk_shift;
+        stop = stop - c < most ? stop : c + most;
+        const int64_t a = (c - first) << chunk_shift;
+        int64_t e = (stop - first) << chunk_shift;
+        e = e < len ? e : len;
         const int64_t n = e > a ? e - a : 0;
         const char *seg = static_cast<const char *>(arena) + (off + a) * kEB;
         bool suspect;
@@ -217,12 +259,15 @@ __global__ void __launch_bounds__(kThreads, 2) static_norms_kernel(const void *a
         if (suspect)
             x = gnmr::warp_segment_sumsq_f64<DT>(seg, n, lane);
         s += x;
+        c = stop;
     }
     finish(b, wp, s);
+    write_pending();
 }
 
 std::mutex g_setup_mu;
 void *g_scratch_addr[kMaxDevices] = {};
+int g_sms[kMaxDevices] = {};
 
 // The host computes each call's chunk and slot tables into these static
 // arrays (no allocation) and copies them to the device scratch; the copy
@@ -248,41 +293,44 @@ struct Uploaded {
     int32_t num_units = 0;
     int64_t chunks = 0;
     int64_t warps = 0;
+    bool split = false;                  // some unit is shared by several warps
+    int64_t max_end = 0;                 // end of the last unit that is not empty,
+    int64_t reach = 0;                   // of any unit,
+    int64_t longest = 0;                 // and the longest length
     int64_t offsets[kMaxUnits];
     int64_t lengths[kMaxUnits];
 };
 Uploaded g_uploaded;
 unsigned long long g_next_generation = 1;   // the device scratch starts at 0: no layout
 
-bool same_layout(int dev, int sms, int32_t dtype, int32_t num_units, const int64_t *offsets,
-                 const int64_t *lengths)
+bool same_units(int32_t num_units, const int64_t *offsets, const int64_t *lengths)
 {
     const Uploaded &u = g_uploaded;
-    return u.device == dev && u.sms == sms && u.dtype == dtype && u.num_units == num_units &&
+    return u.device >= 0 && u.num_units == num_units &&
            std::memcmp(u.offsets, offsets, sizeof(int64_t) * num_units) == 0 &&
            std::memcmp(u.lengths, lengths, sizeof(int64_t) * num_units) == 0;
 }
 
-// Device address of g_norm_scratch on the current device.  In host code the
-// name g_norm_scratch is only a host-side stand-in, so the address is looked
-// up once per device, with that device current, and cached.
-cudaError_t scratch_address(void **out)
+// Device address of g_norm_scratch on the current device, and its SM count.  In
+// host code the name g_norm_scratch is only a host-side stand-in, so the address
+// is looked up once per device, with that device current, and cached.
+cudaError_t scratch_address(int dev, void **out, int *sms)
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess)
-        return e;
     if (dev < 0 || dev >= kMaxDevices)
         return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_setup_mu);
     if (!g_scratch_addr[dev]) {
         void *p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_norm_scratch);
+        *sms = 0;
+        if (cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || g_sms[dev] < 1)
+            return cudaSuccess;                             // the caller reports it by *sms
+        const cudaError_t e = cudaGetSymbolAddress(&p, g_norm_scratch);
         if (e != cudaSuccess)
             return e;
         g_scratch_addr[dev] = p;
     }
     *out = g_scratch_addr[dev];
+    *sms = g_sms[dev];
     return cudaSuccess;
 }
 
@@ -320,34 +368,48 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
     if (!offsets || !lengths || !d_norms || arena_elems < 0)
         return reject(GNMR_ERR_INVALID_ARG, kErrNull);
     const int eb = dtype == GNMR_DTYPE_BF16 ? 2 : 4;
-    const int chunk_shift = eb == 2 ? 15 : 14;             // 64 KiB chunks
-    const int64_t chunk_elems = int64_t(1) << chunk_shift;
-    static_assert(kChunkBytes == (int64_t(1) << 16), "chunk_shift assumes 64 KiB chunks");
-    int64_t max_end = 0;
-    for (int32_t b = 0; b < num_units; ++b) {
-        const int64_t o = offsets[b], l = lengths[b];
-        if (o < 0 || l < 0 || o > arena_elems - l)
+    std::lock_guard<std::mutex> lock(g_plan_mu);
+    // The units of the layout last uploaded were checked when they were new; of
+    // them only the arena's size is checked again.
+    const bool known = same_units(num_units, offsets, lengths);
+    int64_t max_end = 0, reach = 0, longest = 0;
+    if (known) {
+        if (g_uploaded.reach > arena_elems)
             return reject(GNMR_ERR_LAYOUT, kErrLayout);
-        if (l > 0 && o + l > max_end)
-            max_end = o + l;
+        max_end = g_uploaded.max_end;
+        reach = g_uploaded.reach;
+        longest = g_uploaded.longest;
+    } else {
+        for (int32_t b = 0; b < num_units; ++b) {
+            const int64_t o = offsets[b], l = lengths[b];
+            if (o < 0 || l < 0 || o > arena_elems - l)
+                return reject(GNMR_ERR_LAYOUT, kErrLayout);
+            reach = o + l > reach ? o + l : reach;
+            if (l > 0 && o + l > max_end)
+                max_end = o + l;
+            longest = l > longest ? l : longest;
+        }
     }
+    const int bytes_shift = longest > (int64_t(1) << kCoarseShift) / eb ? kFineShift : kCoarseShift;
+    const int64_t chunk_bytes = int64_t(1) << bytes_shift;
+    const int chunk_shift = bytes_shift - (eb == 2 ? 1 : 2);   // in elements
     if ((!d_arena && max_end > 0) || reinterpret_cast<uintptr_t>(d_arena) % eb != 0)
         return reject(GNMR_ERR_INVALID_ARG, kErrArena);
 
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess)
+        return reject(GNMR_ERR_CUDA, kErrDevice);
     void *addr = nullptr;
-    cudaError_t e = scratch_address(&addr);
+    cudaError_t e = scratch_address(dev, &addr, &sms);
     if (e != cudaSuccess)
         return reject(GNMR_ERR_CUDA, kErrCuda);
+    if (sms < 1)
+        return reject(GNMR_ERR_CUDA, kErrDevice);
     unsigned char *base = static_cast<unsigned char *>(addr);
     const View v = carve(base);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return reject(GNMR_ERR_CUDA, kErrDevice);
 
-    std::lock_guard<std::mutex> lock(g_plan_mu);
-    if (!same_layout(dev, sms, dtype, num_units, offsets, lengths)) {
+    if (!known || g_uploaded.device != dev || g_uploaded.sms != sms || g_uploaded.dtype != dtype) {
         g_uploaded.device = -1;                             // until the uploads are enqueued
         int64_t T = 0, total = 0;
         for (int32_t b = 0; b < num_units; ++b) {
@@ -369,9 +431,9 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
                 const int64_t t = total / want * k + total % want * k / want;
                 if (t >= uend)
                     break;
-                // chunk j >= 1 of b starts at cost ucost + kUnitCostBytes + j * kChunkBytes
+                // chunk j >= 1 of b starts at cost ucost + kUnitCostBytes + j * chunk_bytes
                 const int64_t r = t - ucost - gnmr::kUnitCostBytes;
-                const int64_t j = t <= ucost ? 0 : (r <= kChunkBytes ? 1 : (r + kChunkBytes - 1) / kChunkBytes);
+                const int64_t j = t <= ucost ? 0 : (r <= chunk_bytes ? 1 : (r + chunk_bytes - 1) / chunk_bytes);
                 const int64_t c = j < nch ? g_host_chunk_start[b] + j : g_host_chunk_start[b + 1];
                 if (c > g_host_bound[nb - 1])
                     g_host_bound[nb++] = c;
@@ -382,6 +444,7 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
             g_host_bound[nb++] = T;
         const int64_t W = nb - 1;
         int64_t slot = 0, wi = 0;
+        bool split = false;
         for (int32_t b = 0; b < num_units; ++b) {
             const int64_t first = g_host_chunk_start[b], last = g_host_chunk_start[b + 1] - 1;
             while (g_host_bound[wi + 1] <= first)
@@ -391,6 +454,7 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
                 ++wj;
             g_host_part_base[b] = slot;
             slot += wj - wi + 1;
+            split |= wj > wi;
             g_host_pieces[b] = static_cast<int64_t>(static_cast<uint64_t>(wi) | (static_cast<uint64_t>(wj - wi + 1) << 32));
         }
         int32_t u = 0;                                      // unit of each warp's first chunk
@@ -434,18 +498,35 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
         g_uploaded.num_units = num_units;
         g_uploaded.chunks = T;
         g_uploaded.warps = W;
+        g_uploaded.split = split;
+        g_uploaded.max_end = max_end;
+        g_uploaded.reach = reach;
+        g_uploaded.longest = longest;
     }
     const int64_t W = g_uploaded.warps;
-    e = cudaMemsetAsync(v.ticket, 0, sizeof(uint32_t) * num_units, st);
+    // Both kernels are launched as programmatic dependents of what precedes
+    // them on the stream, and wait for it to complete before they touch memory.
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (g_uploaded.split) {
+        const int64_t clear = (num_units + kThreads - 1) / kThreads;
+        cfg.gridDim = dim3(static_cast<unsigned>(clear < sms ? clear : sms));
+        e = cudaLaunchKernelEx(&cfg, clear_tickets_kernel, v.ticket, num_units);
+    }
+    if (e == cudaSuccess) {
+        cfg.gridDim = dim3(static_cast<unsigned>((W + kWarpsPerCta - 1) / kWarpsPerCta));
+        const unsigned long long gen = g_uploaded.generation;
+        e = cudaLaunchKernelEx(&cfg, dtype == GNMR_DTYPE_BF16 ? static_norms_kernel<1> : static_norms_kernel<0>, d_arena,
+                               base, num_units, W, chunk_shift, d_norms, gen);
+    }
     if (e != cudaSuccess)
-        return reject(GNMR_ERR_CUDA, kErrCuda);
-    const int grid = static_cast<int>((W + kWarpsPerCta - 1) / kWarpsPerCta);
-    const unsigned long long gen = g_uploaded.generation;
-    if (dtype == GNMR_DTYPE_BF16)
-        static_norms_kernel<1><<<grid, kThreads, 0, st>>>(d_arena, base, num_units, W, chunk_elems, d_norms, gen);
-    else
-        static_norms_kernel<0><<<grid, kThreads, 0, st>>>(d_arena, base, num_units, W, chunk_elems, d_norms, gen);
-    e = cudaGetLastError();
+        cudaGetLastError();                                 // reported here, not by the caller's next call
     if (e != cudaSuccess)
         return reject(GNMR_ERR_CUDA, kErrCuda);
     return GNMR_OK;

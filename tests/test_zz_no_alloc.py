@@ -157,3 +157,38 @@ def test_static_norms_reject_tables_of_another_layout(cuda_device):
     s1.synchronize()
     np.testing.assert_allclose(out2.cpu().numpy(), oracle.unit_norms(host, off2, ln2), rtol=RTOL, atol=0)
     assert np.isnan(out1.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("name", ["uncut", "cut", "spans", "many"])
+def test_static_norms_of_cut_and_uncut_units(dtype, name, cuda_device):
+    """Units up to 16 KiB are never cut (no tickets), longer ones at 4 KiB and
+    summed 64 KiB at a time; a warp finishes more units than its 32 lanes
+    hold.  The same layout again on a shorter arena is rejected, and in the
+    other dtype planned anew."""
+    import torch
+    lib = N.load()
+    top = (16 << 10) // (4 if dtype == "f32" else 2)
+    rng = np.random.default_rng(3)
+    ln = {"uncut": rng.integers(0, top + 1, 3000), "cut": np.append(rng.integers(0, top, 500), [top + 1, top, top - 1]),
+          "spans": np.array([0, 4 * top, 4 * top + 1, 40_000_003, 1, 8 * top - 1, 3]),
+          "many": rng.integers(0, 3, 131072)}[name].astype(np.int64)
+    off = np.concatenate([[0], np.cumsum(ln)[:-1]]).astype(np.int64) + 1
+    n = int(ln.sum()) + 1
+    ids = torch.repeat_interleave(torch.arange(len(ln), device=cuda_device), torch.from_numpy(ln).to(cuda_device))
+    out = torch.empty(len(ln), dtype=torch.float64, device=cuda_device)
+
+    def call(arena, elems):
+        code = N.GNMR_DTYPE_BF16 if arena.dtype == torch.bfloat16 else N.GNMR_DTYPE_F32
+        return lib.gnmr_unit_norms_static(arena.data_ptr(), elems, code, len(ln), off.ctypes.data, ln.ctypes.data,
+                                          out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+
+    for seed, dt in enumerate([dtype, dtype, "bf16" if dtype == "f32" else "f32"]):
+        g = torch.Generator(cuda_device).manual_seed(seed)
+        arena = torch.randn(n, device=cuda_device, generator=g).to(torch.bfloat16 if dt == "bf16" else torch.float32)
+        out.fill_(float("nan"))
+        assert call(arena, n) == N.GNMR_OK, N.last_error(None)
+        want = torch.zeros(len(ln), dtype=torch.float64, device=cuda_device).index_add_(0, ids, arena[1:].double().square())
+        # fp32 roundings of one piece, as in the step kernel's tests
+        torch.testing.assert_close(out, want.sqrt(), rtol=1e-6, atol=0)
+        assert call(arena, n - 1) == N.GNMR_ERR_LAYOUT and N.last_error(None) == "unit off arena"
