@@ -5,9 +5,10 @@
 // A warp reads a segment with 16-byte loads (no L1 allocation, 256-byte L2
 // prefetch), squares in fp32, sums short blocks in
 // fp32 and the blocks as an unevaluated pair of floats (hi + lo, about 48
-// significant bits), then adds the 32 lanes' totals with an fp32 xor
-// butterfly (non-negative terms: at most five roundings, about 3e-7
-// relative) and converts to fp64 once per segment.  It flags segments whose fp32 squares
+// significant bits), then adds the 32 lanes' totals in fixed point (exact from
+// the lanes' rounding to 26 bits on; a five-level fp32 tree over the lanes was
+// up to 3e-7 off) and forms the fp64 result once per segment.  It flags
+// segments whose fp32 squares
 // may have lost accuracy (denormal or overflowing squares), which the caller
 // recomputes with exact fp64 squares.  Any element alignment: a scalar head
 // and tail around the 16-byte body.
@@ -17,9 +18,8 @@
 // warps.  A five-round fp64 shuffle reduction per segment held that pipe 40 %
 // of the time on layouts of many small units and stalled the streams; the
 // fp32 error-free additions run on the fp32 pipe.  The pairs keep a long run
-// of blocks accurate; the final five-level tree over the lanes does not need
-// them (measured: a pair-wise TwoSum butterfly there cost 1 us more on 100K
-// units).
+// of blocks accurate.  The lanes' sum is three warp reductions of integers
+// (redux), with no fp64 instruction at all.
 #ifndef GNMR_STREAM_CUH
 #define GNMR_STREAM_CUH
 
@@ -149,8 +149,8 @@ __device__ __forceinline__ void pair_add(float &hi, float &lo, float x)
 
 // Sum of squares of n elements at seg, by the whole warp.  Returns the sum
 // in every lane and sets `suspect` when fp32 squaring may have lost accuracy:
-// a nonzero segment whose sum is below 2^-100 (denormal squares) or above
-// 2^100 (possible fp32 overflow), or a NaN/Inf sum.
+// a nonzero segment whose largest lane total is below 2^-100 (denormal squares),
+// at least 2^100 (possible fp32 overflow), or NaN or Inf.
 template <int DT, int kUnroll>
 __device__ __forceinline__ double warp_segment_sumsq(const char *seg, int64_t n, int lane,
                                                      bool &suspect)
@@ -221,16 +221,26 @@ __device__ __forceinline__ double warp_segment_sumsq(const char *seg, int64_t n,
         blk += a;
     }
     pair_add(acc_hi, acc_lo, blk);
-    // the lanes' totals (non-negative) summed by an fp32 xor butterfly: both
-    // partners add the same two operands, so every lane ends with the same bits
-    float tot = acc_hi + acc_lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        tot += __shfl_xor_sync(kFull, tot, o);
-    const float lead = tot;
-    const double acc = static_cast<double>(tot);
-    bits = __reduce_or_sync(kFull, bits);
-    suspect = (bits & Elem<DT>::kMagnitude) != 0u && !(lead >= 0x1p-100f && lead <= 0x1p+100f);
+    // The lanes' totals (non-negative) added as 26-bit fractions of twice the
+    // largest one's power of two: the integer sum is exact and the same in every
+    // lane, and a lane's rounding to its fraction is at most 2^-26 of the largest
+    // total.  As fast as a five-level fp32 xor tree, whose error it cuts from 1-3e-8
+    // to 2-7e-9 (norms of a whole layout against 64 bits).
+    const uint32_t tot = __float_as_uint(acc_hi + acc_lo);
+    const uint32_t e = __reduce_max_sync(kFull, tot) >> 23;                    // > 254 for NaN and Inf
+    suspect = false;
+    if (e - 27u >= 200u) {                                // the largest not in [2^-100, 2^100)
+        suspect = (__reduce_or_sync(kFull, bits) & Elem<DT>::kMagnitude) != 0u;
+        return 0.0;
+    }
+    const uint32_t own = tot >> 23;
+    const uint32_t sh = min(e - own, 27u);
+    const uint32_t frac = own ? ((tot & 0x7fffffu) | 0x800000u) << 2 : 0u;     // 26 bits
+    const uint32_t sum = __reduce_add_sync(kFull, (frac + ((1u << sh) >> 1)) >> sh);
+    // sum * 2^(e - 152) in binary64, put together on the integer pipe
+    const uint32_t lz = __clz(sum);
+    const uint32_t m = sum << (lz + 1);
+    const double acc = __hiloint2double(static_cast<int>(((902u + e - lz) << 20) | (m >> 12)), static_cast<int>(m << 20));
     return acc;
 }
 

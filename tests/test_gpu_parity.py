@@ -778,3 +778,28 @@ def test_block_loop_layouts(name, dtype, cuda_device):
             # a piece's fp32 sum: at most about 27 roundings of 2^-24 per block
             # of 16 iterations and 5 over the lanes, halved by the square root
             torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("shape", ["small", "large"])
+@pytest.mark.parametrize("power", [-75, -51, -50, -49, -3, 0, 40, 48, 49, 50, 51, 62])
+def test_lane_totals_of_any_size(power, shape, cuda_device):
+    """The warp's sum over lanes whose totals differ by up to 2^60, around the
+    ends of the range beyond which squares are taken in fp64."""
+    import torch
+    lengths = np.array([1, 31, 128, 129, 1000, 4096, 20_000, 300_001], np.int64)
+    offsets = np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64)
+    n = int(lengths.sum())
+    g = torch.Generator(cuda_device).manual_seed(5)
+    for spread in (0, 4, 30):
+        x = torch.randn(n, device=cuda_device, generator=g, dtype=torch.float64)
+        x = x * torch.exp2(-spread * torch.rand(n, device=cuda_device, generator=g, dtype=torch.float64)) * 2.0 ** power
+        arena = x.float()
+        with Monitor(offsets, lengths, dtype="f32", loop_shape=shape) as mon:
+            stats = mon.new_stats()
+            mon.step(arena, stats=stats)
+            got = stats["norm"].cpu().numpy()
+        want = [float(arena[o:o + m].double().square().sum().sqrt()) for o, m in zip(offsets.tolist(), lengths.tolist())]
+        # in a block of 16 iterations of up to 16 vectors at most 27 fp32 roundings
+        # of non-negative terms, and 2^-26 of the largest lane 32 times; the root
+        # halves it: 27 / 2 * 2^-24 + 16 * 2^-26 < 1.1e-6
+        np.testing.assert_allclose(got, want, rtol=1.1e-6, atol=0)
