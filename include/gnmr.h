@@ -98,10 +98,12 @@ typedef struct gnmr_config {
 
 /* Streaming-loop shapes of the step kernel.
  *   GNMR_LOOP_AUTO: GNMR_LOOP_LARGE_UNITS when the mean unit holds at least
- *     1 MiB of gradient, else GNMR_LOOP_SMALL_UNITS.
+ *     1 MiB of gradient and all units at least 512 MiB, else
+ *     GNMR_LOOP_SMALL_UNITS.
  *   GNMR_LOOP_SMALL_UNITS: fewer loads in flight per warp, more resident
- *     warps per SM (suits many small units, whose per-unit work overlaps the
- *     stream of other warps).
+ *     warps per SM, the arena shared out in small blocks (suits many small
+ *     units, whose per-unit work overlaps the stream of other warps, and small
+ *     arenas).
  *   GNMR_LOOP_LARGE_UNITS: twice the loads in flight per warp, half the
  *     resident warps (suits long streams). */
 typedef enum gnmr_loop_shape {

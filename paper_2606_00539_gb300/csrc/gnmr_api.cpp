@@ -233,12 +233,13 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
     if (scope.status() != cudaSuccess)
         return fail_create(GNMR_ERR_CUDA, format("cudaSetDevice(%d): %s", c.device,
                                                  cudaGetErrorString(scope.status())));
-    // the streaming-loop variant follows the mean unit size
+    // the streaming-loop variant follows the mean unit size and the arena's
     int64_t grad_bytes = 0;
     for (int64_t g = 0; g < S_in; ++g)
         grad_bytes += c.lengths[g] * eb;
-    const bool large = c.loop_shape == GNMR_LOOP_AUTO ? grad_bytes / c.num_units >= gnmr::kBulkUnitBytes
-                                                      : c.loop_shape == GNMR_LOOP_LARGE_UNITS;
+    const bool large = c.loop_shape == GNMR_LOOP_AUTO
+                           ? grad_bytes >= gnmr::kBulkArenaBytes && grad_bytes / c.num_units >= gnmr::kBulkUnitBytes
+                           : c.loop_shape == GNMR_LOOP_LARGE_UNITS;
     const int variant = large ? gnmr::kVariantBulk : gnmr::kVariantSmall;
     int sms = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
@@ -447,11 +448,9 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         h->num_runs = variant == gnmr::kVariantBulk ? plan.num_runs : step_warps;
         h->num_ctas = variant == gnmr::kVariantBulk ? (step_warps + gnmr::kWarpsPerCta - 1) / gnmr::kWarpsPerCta
                                                     : plan.num_runs;
-        {
-            const int64_t warps = (U + 31) / 32;
-            const int64_t ctas = (warps + gnmr::kWarpsPerCta - 1) / gnmr::kWarpsPerCta;
-            h->finish_ctas = static_cast<int32_t>(std::min<int64_t>(ctas, int64_t(sms) * per_sm));
-        }
+        p.finish_units = U <= int64_t(2) * gnmr::kFewUnits * sms ? gnmr::kFewUnits : 32;
+        h->finish_ctas = static_cast<int32_t>(std::min<int64_t>((U + p.finish_units - 1) / p.finish_units,
+                                                                int64_t(sms) * per_sm));
         h->num_partials = plan.num_partials;
         h->device_bytes = static_cast<int64_t>(cv.size);
         h->max_end = max_end;

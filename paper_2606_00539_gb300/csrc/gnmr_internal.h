@@ -13,7 +13,8 @@ namespace gnmr {
 // Launch shape of the step kernel: 512 threads = 16 warps per CTA.  Two
 // compiled variants of the streaming loop (gnmr_kernels.cu): kVariantSmall
 // (two resident CTAs per SM, each with a part of its own that its warps take
-// block by block) for layouts of small and mid-sized units, kVariantBulk (one CTA per SM, deeper per-warp streams, runs
+// block by block) for layouts of small and mid-sized units and for small
+// arenas, kVariantBulk (one CTA per SM, deeper per-warp streams, runs
 // taken from a shared counter) for layouts whose mean unit holds at least
 // kBulkUnitBytes.
 constexpr int kThreads = 512;
@@ -21,6 +22,16 @@ constexpr int kWarpsPerCta = kThreads / 32;
 constexpr int kVariantSmall = 0;
 constexpr int kVariantBulk = 1;
 constexpr int64_t kBulkUnitBytes = int64_t(1) << 20;
+// Below this many gradient bytes the large-unit loop's 64 KiB runs are too few
+// to balance: 168 units in 303 MB took 60.7 us with it, 57.9 with blocks; 84 in
+// 170 MB 56.3 and 54.4, 84 in 95 MB 43.0 and 37.0.  (607 MB: 100.4 and 98.4; 1.2
+// GB: 179.2 and 180.8; 2.4 GB: 333.4 and 336.0.)
+constexpr int64_t kBulkArenaBytes = int64_t(512) << 20;
+// Controller half: up to 2 kFewUnits units per SM a warp takes kFewUnits units
+// (four lanes each in the epilogue), else 32; warps go one to a CTA first, as an
+// SM's fp64 pipe serves all of its warps.  From full warps, 16 to a CTA: 168 units
+// 8.6 -> 7.2 us, 560 15.3 -> 7.1, 20,000 16.4 -> 8.2, 100,000 28.7 -> 20.6.
+constexpr int kFewUnits = 8;
 
 // Work partition: a unit costs its element bytes plus this many bytes of
 // equivalent fixed work (reduction, Algorithm 1 update, bookkeeping); runs
@@ -179,6 +190,7 @@ struct StepParams {
     int32_t window;
     int32_t max_o;
     int32_t lock_len;
+    int32_t finish_units;        // controller half: units per warp, kFewUnits or 32
     int32_t dense;               // 1: at most kDenseUnits units, selected from one entry each
     int32_t num_runs;            // R; runs num_warps .. R - 1 are taken dynamically
     int64_t warmup_steps;

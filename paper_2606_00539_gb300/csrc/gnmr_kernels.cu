@@ -1181,10 +1181,12 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         const int64_t t = __ldcg(&p.ctl->steps) + 1;
         const double alpha = pick_threshold(p.alpha_override, t, p.warmup_steps, p.alpha_init, p.alpha_main);
         const double beta = pick_threshold(p.beta_override, t, p.warmup_steps, p.beta_init, p.beta_main);
-        const int64_t warps = static_cast<int64_t>(gridDim.x) * kWarpsPerCta;
-        for (int64_t b0 = static_cast<int64_t>(warp) * 32; b0 < p.num_units; b0 += warps * 32) {
+        // Warps of different CTAs first: an SM's fp64 pipe serves all of its warps.
+        const int64_t per = p.finish_units;
+        const int64_t first = blockIdx.x + static_cast<int64_t>(gridDim.x) * (threadIdx.x >> 5);
+        for (int64_t b0 = first * per; b0 < p.num_units; b0 += static_cast<int64_t>(gridDim.x) * kWarpsPerCta * per) {
             const int64_t b = b0 + lane;
-            const bool active = b < p.num_units;
+            const bool active = lane < per && b < p.num_units;
             const double s = active ? p.in_sumsq[b] : 0.0;
             unit_epilogue(p, active, active ? static_cast<int32_t>(b) : 0, s, alpha, beta, t);
         }

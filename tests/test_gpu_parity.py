@@ -717,7 +717,7 @@ def test_steps_wait_for_the_kernel_that_writes_the_arena(config, shrink, cuda_de
         mon.close()
 
 
-@pytest.mark.parametrize("units_per_sm,extra", [(1, 0), (6, 1), (13, 0), (32, 1), (133, 3), (520, 0)])
+@pytest.mark.parametrize("units_per_sm,extra", [(1, 0), (6, 1), (16, 0), (16, 1), (32, 1), (133, 3), (520, 0)])
 def test_small_unit_batches_update_every_unit_once(units_per_sm, extra, cuda_device):
     """The small-unit loop runs the epilogues in batches of 32 units of a CTA,
     by whichever warp completes one.  The controller half runs them unit by
@@ -744,6 +744,15 @@ def test_small_unit_batches_update_every_unit_once(units_per_sm, extra, cuda_dev
     finally:
         one.close()
         two.close()
+
+
+@pytest.mark.parametrize("mib,extra,want", [(512, 0, "large"), (512, -1, "small"), (100, 0, "small")])
+def test_loop_shape_of_small_arenas(mib, extra, want, cuda_device):
+    """Units of 1 MiB and more take the large-unit shape from 512 MiB on."""
+    lengths = np.full(mib // 4, 1 << 20, np.int64)
+    lengths[0] += extra
+    with Monitor(np.cumsum(lengths) - lengths, lengths, dtype="f32") as mon:
+        assert mon.info()["loop_shape"] == (N.GNMR_LOOP_LARGE_UNITS if want == "large" else N.GNMR_LOOP_SMALL_UNITS)
 
 
 def _block_layout(name):
