@@ -244,7 +244,7 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
     int sms = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
     if (e == cudaSuccess)
-        e = gnmr::step_occupancy(c.dtype, variant, &per_sm);
+        e = gnmr::step_occupancy(c.dtype, variant, c.num_units <= gnmr::kDenseUnits, &per_sm);
     if (e != cudaSuccess || sms < 1 || per_sm < 1)
         return fail_create(GNMR_ERR_CUDA, format("device query failed: %s", cudaGetErrorString(e)));
 

@@ -61,6 +61,11 @@ constexpr int kBlocksPerCta = 2048;
 constexpr int64_t kMinCtaBytes = int64_t(24) << 10;
 constexpr int64_t kMinBlockBytes = int64_t(8) << 10;
 constexpr int64_t kMaxBlockBytes = int64_t(1) << 20;
+// Arenas of at most kSmallArenaCtaBytes of cost per resident CTA are cut between
+// units: joining the parts of a split unit takes longer than streaming a unit of
+// up to kWholeUnitBytes, 8 KiB a warp (64 units in 3.7 MB: 11.4 -> 10.1 us).
+constexpr int64_t kSmallArenaCtaBytes = int64_t(48) << 10;
+constexpr int64_t kWholeUnitBytes = int64_t(128) << 10;
 
 // A piece of one segment.
 struct alignas(16) Block {
@@ -208,8 +213,8 @@ constexpr int kStepFinish = 2;
 cudaError_t launch_step(const StepParams &p, int dtype, int num_ctas, cudaStream_t stream,
                         int mode = kStepFull, int variant = kVariantSmall);
 
-// Resident CTAs per SM of the step kernel for `dtype` and `variant`.
-cudaError_t step_occupancy(int dtype, int variant, int *ctas_per_sm);
+// Resident CTAs per SM of the step kernel for `dtype`, `variant` and `dense`.
+cudaError_t step_occupancy(int dtype, int variant, bool dense, int *ctas_per_sm);
 
 // Records the failure detail that gnmr_last_error(NULL) reports on the
 // calling thread (used by calls that have no handle).
@@ -228,10 +233,11 @@ struct Plan {
 
 // Segments must be grouped by unit (seg_unit non-decreasing, every unit
 // 0..num_units-1 present).  Cuts the stream into at most max_runs runs, none
-// smaller than kMinRunBytes unless the whole problem is.  Returns false if
-// the inputs are out of range.
+// smaller than kMinRunBytes unless the whole problem is; or at the given costs
+// (increasing).  Returns false if the inputs are out of range.
 bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int32_t *seg_unit,
-                    int32_t num_units, int elem_bytes, int32_t max_runs, Plan &out);
+                    int32_t num_units, int elem_bytes, int32_t max_runs, Plan &out,
+                    const std::vector<int64_t> *targets = nullptr);
 
 // The blocks of a plan with one run per CTA (small-unit loop).
 struct BlockPlan {

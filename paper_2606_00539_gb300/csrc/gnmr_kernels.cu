@@ -19,7 +19,8 @@
 // be shared with other CTAs.  The plan is read before the grid's programmatic
 // wait.  One GB300, from one run per warp to blocks: 100K fp32 units 263.3 ->
 // 243.1 us; 30,000 short bf16 units 34.2 -> 32.2 us; 560 units in 125 MB 30.7
-// -> 30.0 us; 64 units in 3.7 MB 11.0 -> 11.4 us.
+// -> 30.0 us; 64 units in 3.7 MB 11.0 -> 9.4 us, with whole units per CTA and
+// the state read ahead.
 //
 // Large-unit loop: about 16 runs per warp; each warp starts on its own run and
 // then takes the next untaken one from a global counter, so warps that stream
@@ -168,6 +169,51 @@ __device__ __forceinline__ void append_candidates(const StepParams &p, bool cand
     }
 }
 
+// What the epilogue of up to 32 consecutive units reads, read ahead: the loads
+// and the serial sum of the window (eight fp64 additions of 64 cycles) are 0.8
+// of the 2.9 us between a small step's last sum and its candidates (64 units:
+// 10.1 -> 9.4 us; 560 units in 125 MB: 30.1 -> 29.6).
+struct Preload {
+    UnitState state[kBatch];
+    double window[kBatch];           // sum of the window, oldest to newest (0 if it is not full)
+    uint8_t recoverable[kBatch];
+};
+
+// Sum of a full window, oldest to newest: its loads are issued together.
+__device__ __forceinline__ double window_sum(const double *Q, int w, int head)
+{
+    double q = 0.0;
+    int idx = head, k = 0;
+    for (; k + 8 <= w; k += 8) {
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int ix = idx + j < w ? idx + j : idx + j - w;
+            v[j] = Q[ix];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            q += v[j];
+        idx = idx + 8 < w ? idx + 8 : idx + 8 - w;
+    }
+    for (; k < w; ++k) {
+        q += Q[idx];
+        idx = (idx + 1 == w) ? 0 : idx + 1;
+    }
+    return q;
+}
+
+__device__ __forceinline__ void preload_unit(const StepParams &p, Preload &pre, int32_t b, int slot)
+{
+    const double *Q = p.queue + static_cast<int64_t>(b) * p.window;
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + (p.window - 1)));
+    const UnitState s = p.state[b];
+    pre.recoverable[slot] = p.recoverable[b];
+    pre.state[slot] = s;
+    pre.window[slot] = s.fill == p.window ? window_sum(Q, p.window, s.head) : 0.0;
+}
+
 // Unit epilogue for up to 32 units at once, one per lane (lanes with
 // `active` false only take part in the collective append): Algorithm 1, the
 // combined risk of Sec. 3.3, the statistics outputs and the candidate test of
@@ -181,8 +227,11 @@ __device__ __forceinline__ void append_candidates(const StepParams &p, bool cand
 // each unit four lanes, which do the independent divisions at once: a square
 // root and three rounds of division instead of six (the epilogue of 64 units:
 // 4.4 -> 3.1 us).
-__device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, double sumsq,
-                              double alpha, double beta, int64_t t)
+// pre: nullptr, or what preload_unit() read of units first, first + 1, ...
+template <bool kDense>
+__device__ __forceinline__ void unit_epilogue(const StepParams &p, bool active, int32_t b, double sumsq,
+                                              double alpha, double beta, int64_t t, const Preload *pre = nullptr,
+                                              int32_t first = 0)
 {
     const unsigned mine = __ballot_sync(kFull, active);
     if (!mine)
@@ -209,43 +258,31 @@ __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, doubl
     uint32_t cand_lock = 0;
     // read now, used after the risk: the step's hot-list bin (only the
     // selection, after every CTA, rewrites it)
-    const uint32_t hot_bin = p.dense ? 0u : __ldcg(&p.ctl->hot_bin);
+    const uint32_t hot_bin = kDense ? 0u : __ldcg(&p.ctl->hot_bin);
     UnitState s{};
     double n = 0.0, g = 0.0, d = 0.0, step = 0.0;     // step: the mean's change
     bool rec = false;
     if (active || few) {
-        n = sqrt(sumsq);
         const int w = p.window;
-        double *Q = p.queue + static_cast<int64_t>(b) * w;
-        // the window's lines travel with the state load: the window reads,
-        // which need the state's head, then hit in L1
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + (w - 1)));
-        s = p.state[b];
-        rec = p.recoverable[b] != 0;
-        // mean of the window, summed oldest to newest; its loads are issued
-        // as soon as the state's head is known, before the division for g
-        const bool full = s.fill == w;
         double q = 0.0;
-        if (full) {
-            int idx = s.head, k = 0;
-            for (; k + 8 <= w; k += 8) {
-                double v[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int ix = idx + j < w ? idx + j : idx + j - w;
-                    v[j] = Q[ix];
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    q += v[j];
-                idx = idx + 8 < w ? idx + 8 : idx + 8 - w;
-            }
-            for (; k < w; ++k) {
-                q += Q[idx];
-                idx = (idx + 1 == w) ? 0 : idx + 1;
-            }
+        if (kDense && pre != nullptr) {
+            n = sqrt(sumsq);
+            s = pre->state[b - first];
+            q = pre->window[b - first];
+            rec = pre->recoverable[b - first] != 0;
+        } else {
+            n = sqrt(sumsq);
+            const double *Q = p.queue + static_cast<int64_t>(b) * w;
+            // the window's lines travel with the state load: the window reads,
+            // which need the state's head, then hit in L1
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + (w - 1)));
+            s = p.state[b];
+            rec = p.recoverable[b] != 0;
+            if (s.fill == w)
+                q = window_sum(Q, w, s.head);
         }
+        const bool full = s.fill == w;
         const double count = static_cast<double>(s.count + 1);
         const bool fresh = s.count == 0 || s.mean == 0.0;
         double x, y;
@@ -342,34 +379,35 @@ __device__ void unit_epilogue(const StepParams &p, bool active, int32_t b, doubl
         }
         cand_lock = static_cast<uint32_t>(s.lock) | (s.active ? kCandActive : 0u);
     }
-    if (p.dense) {
+    if constexpr (kDense) {
         // few units: one entry per unit, which the selection reads in full
         if (active) {
             const uint64_t word = static_cast<uint32_t>(cand ? b : -1) | static_cast<uint64_t>(cand_lock) << 32;
             *reinterpret_cast<double2 *>(p.cand + b) = make_double2(r, __longlong_as_double(static_cast<long long>(word)));
         }
-        return;
+    } else {
+        // The capped pool: every candidate, or under the admission cap those not
+        // active at t-1 (the retained ones are selected without ranking).  Pool
+        // members count in the risk histogram; the hot list takes those at or
+        // above this step's predicted bin, and every retained candidate.
+        const bool retained = cand && p.policy == 1 && (cand_lock & kCandActive);
+        bool hot = retained;
+        if (cand && !retained) {
+            const uint32_t bin = risk_bin(risk_key(r));
+            atomicAdd(&p.risk_hist[bin], 1u);
+            hot = bin >= hot_bin;
+        }
+        append_candidates(p, cand, hot, r, b, cand_lock);
     }
-    // The capped pool: every candidate, or under the admission cap those not
-    // active at t-1 (the retained ones are selected without ranking).  Pool
-    // members count in the risk histogram; the hot list takes those at or
-    // above this step's predicted bin, and every retained candidate.
-    const bool retained = cand && p.policy == 1 && (cand_lock & kCandActive);
-    bool hot = retained;
-    if (cand && !retained) {
-        const uint32_t bin = risk_bin(risk_key(r));
-        atomicAdd(&p.risk_hist[bin], 1u);
-        hot = bin >= hot_bin;
-    }
-    append_candidates(p, cand, hot, r, b, cand_lock);
 }
 
 // The same, out of line: the large-unit loop calls it rarely and keeps its
 // registers for the stream.
+template <bool kDense>
 __device__ __noinline__ void unit_epilogue_call(const StepParams &p, bool active, int32_t b, double sumsq,
                                                 double alpha, double beta, int64_t t)
 {
-    unit_epilogue(p, active, b, sumsq, alpha, beta, t);
+    unit_epilogue<kDense>(p, active, b, sumsq, alpha, beta, t);
 }
 
 // A unit of two parts trades its partial through the first slot in one atomic
@@ -909,13 +947,14 @@ __device__ void select_cut(const StepParams &p, bool stat, uint32_t c, uint32_t 
 // With at most kDenseUnits units there are no lists and no histogram: every
 // unit has left one entry, all of them are read at once, and the pool is ranked
 // in shared memory.
+template <bool kDense>
 __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist, uint32_t *misc, double *red,
                                   unsigned char *smem)
 {
     // one round trip for all that the selection starts from
     uint32_t m = 0, n_hot = 0, hot_bin = 0;
     uint4 bins = make_uint4(0u, 0u, 0u, 0u);
-    if (!p.dense) {
+    if (!kDense) {
         m = __ldcg(&p.ctl->n_cand);
         n_hot = __ldcg(&p.ctl->n_hot);
         hot_bin = __ldcg(&p.ctl->hot_bin);
@@ -933,7 +972,7 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
     } else if (stat && t > p.static_warmup + 1) {
         m = 0;
         n_sel = static_cast<uint32_t>(p.static_keep);
-    } else if (p.dense) {
+    } else if (kDense) {
         const uint32_t cap = stat ? static_cast<uint32_t>(p.static_keep) : static_cast<uint32_t>(p.max_o);
         uint64_t *ck = reinterpret_cast<uint64_t *>(smem);
         int32_t *cu = reinterpret_cast<int32_t *>(smem + kCutUnitOffset);
@@ -1075,6 +1114,7 @@ __device__ void select_and_commit(const StepParams &p, int64_t t, uint32_t *hist
 struct BlockShared {
     double sum[kBlocksPerCta];                    // sum of squares of each block
     int32_t unit_end[kBlocksPerCta];              // end of each unit's blocks
+    Preload pre;                                  // of the CTA's last batch
     CtaBlocks cta;
     int32_t left[kBlocksPerCta / kBatch + 2];     // blocks of each batch not yet summed
     int32_t next;                                 // next block to hand out
@@ -1094,9 +1134,10 @@ __device__ __forceinline__ bool batch_sums(const StepParams &p, const BlockShare
     // few units of many blocks: the warp sums each together
     const bool wide = hi - lo > 8 && (units <= 4 || hi - lo > 64);
     s = 0.0;
-    if (!wide)
+    if (!wide) {
         for (int32_t j = lo; j < hi; ++j)
             s += sh.sum[j];
+    }
     for (unsigned m = __ballot_sync(kFull, wide); m; m &= m - 1) {
         const int l = __ffs(m) - 1;
         const int32_t j0 = __shfl_sync(kFull, lo, l), j1 = __shfl_sync(kFull, hi, l);
@@ -1130,7 +1171,8 @@ __device__ __forceinline__ bool batch_sums(const StepParams &p, const BlockShare
 // sum of squares written to out_sumsq (the first half of a sharded step).
 // kStepFinish: no gradient read; phases 2-3 on the sums in in_sumsq (the
 // second half, after the caller has reduced the shards' sums).
-template <int DT, int MODE, int V>
+// kDense: at most kDenseUnits units (one entry each for the selection, no lists).
+template <int DT, int MODE, int V, bool kDense>
 __global__ void __launch_bounds__(kThreads, Shape<V>::kMinCtas)
 gnmr_step_kernel(const __grid_constant__ StepParams p)
 {
@@ -1159,7 +1201,9 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         for (int32_t k = threadIdx.x; k * kBatch < units; k += kThreads) {
             const int32_t u0 = unit + k * kBatch, n = units - k * kBatch;
             const int32_t b0 = p.unit_block[u0] - first_block, b1 = p.unit_block[u0 + (n < kBatch ? n : kBatch)] - first_block;
-            sh.left[k] = (b1 < blocks ? b1 : blocks) - (b0 > 0 ? b0 : 0);
+            // the last batch also waits for what its epilogue reads ahead
+            const bool last = MODE == kStepFull && kDense && n <= kBatch;
+            sh.left[k] = (b1 < blocks ? b1 : blocks) - (b0 > 0 ? b0 : 0) + (last ? 1 : 0);
         }
         if (threadIdx.x == 0) {
             sh.next = kWarpsPerCta;
@@ -1188,7 +1232,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             const int64_t b = b0 + lane;
             const bool active = lane < per && b < p.num_units;
             const double s = active ? p.in_sumsq[b] : 0.0;
-            unit_epilogue(p, active, active ? static_cast<int32_t>(b) : 0, s, alpha, beta, t);
+            unit_epilogue<kDense>(p, active, active ? static_cast<int32_t>(b) : 0, s, alpha, beta, t);
         }
     } else if (Shape<V>::kBlocks) {
         // t, alpha_t and beta_t are fixed for the whole step.
@@ -1196,8 +1240,25 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         const double alpha = pick_threshold(p.alpha_override, t, p.warmup_steps, p.alpha_init, p.alpha_main);
         const double beta = pick_threshold(p.beta_override, t, p.warmup_steps, p.beta_init, p.beta_main);
         const char *arena = static_cast<const char *>(p.arena);
-        // The state of the CTA's last batch of units, whose epilogue nothing hides.
-        if (MODE == kStepFull && threadIdx.x < kBatch && static_cast<int32_t>(threadIdx.x) < sh.cta.units) {
+        // A warp that completes a batch runs it only when it has no block in
+        // hand: a block kept waiting for an epilogue would hold up its own batch.
+        int32_t i = threadIdx.x >> 5, batch = -1;
+        const int32_t last_batch = (sh.cta.units - 1) / kBatch;
+        auto run_batch = [&](int32_t k) {
+            int32_t u;
+            double sumsq;
+            const bool active = batch_sums(p, sh, k, u, sumsq, lane);
+            if (MODE == kStepPartials) {
+                if (active)
+                    p.out_sumsq[u] = sumsq;
+            } else {
+                unit_epilogue<kDense>(p, active, u, sumsq, alpha, beta, t, kDense && k == last_batch ? &sh.pre : nullptr,
+                                      sh.cta.unit + k * kBatch);
+            }
+        };
+        // Nothing hides the last batch's epilogue.  With few units the last warp
+        // reads ahead what that needs beside the sums; else its lines are fetched.
+        if (MODE == kStepFull && !kDense && threadIdx.x < kBatch && static_cast<int32_t>(threadIdx.x) < sh.cta.units) {
             const int32_t u = sh.cta.unit + sh.cta.units - 1 - static_cast<int32_t>(threadIdx.x);
             const double *Q = p.queue + static_cast<int64_t>(u) * p.window;
             asm volatile("prefetch.global.L1 [%0];" ::"l"(p.state + u));
@@ -1205,30 +1266,41 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             asm volatile("prefetch.global.L1 [%0];" ::"l"(Q));
             asm volatile("prefetch.global.L1 [%0];" ::"l"(Q + p.window - 1));
         }
-        // A warp that completes a batch runs it only when it has no block in
-        // hand: a block kept waiting for an epilogue would hold up its own batch.
-        int32_t i = threadIdx.x >> 5, batch = -1;
-        while (i < blocks) {
-            // the next block's index and table entry travel under this one's stream
-            int32_t next = blocks;
-            if (batch < 0) {
-                if (lane == 0)
-                    next = atomicAdd(&sh.next, 1);
-                next = __shfl_sync(kFull, next, 0);
-            }
-            const Block follow = p.block[first_block + (next < blocks ? next : i)];
-            const char *seg = arena + cur.start * kEB;
-            bool suspect;
-            double s = warp_segment_sumsq<DT, Shape<V>::kUnroll>(seg, cur.elems, lane, suspect);
-            if (suspect)
-                s = warp_segment_sumsq_f64<DT>(seg, cur.elems, lane);
+        if (MODE == kStepFull && kDense && i == kWarpsPerCta - 1) {
+            if (last_batch * kBatch + lane < sh.cta.units)
+                preload_unit(p, sh.pre, sh.cta.unit + last_batch * kBatch + lane, lane);
+            __threadfence_block();
+            __syncwarp();
             int32_t left = 0;
-            if (lane == 0) {
-                sh.sum[i] = s;
-                __threadfence_block();
-                left = atomicSub(&sh.left[cur.batch], 1);
+            if (lane == 0)
+                left = atomicSub(&sh.left[last_batch], 1);
+            if (__shfl_sync(kFull, left, 0) == 1)        // every block was summed before
+                batch = last_batch;
+        }
+        while (i < blocks || (kDense && batch >= 0)) {
+            int32_t next = blocks, done = -1;
+            Block follow = cur;
+            if (!kDense || i < blocks) {
+                // the next block's index and table entry travel under this one's stream
+                if (batch < 0) {
+                    if (lane == 0)
+                        next = atomicAdd(&sh.next, 1);
+                    next = __shfl_sync(kFull, next, 0);
+                }
+                follow = p.block[first_block + (next < blocks ? next : i)];
+                const char *seg = arena + cur.start * kEB;
+                bool suspect;
+                double s = warp_segment_sumsq<DT, Shape<V>::kUnroll>(seg, cur.elems, lane, suspect);
+                if (suspect)
+                    s = warp_segment_sumsq_f64<DT>(seg, cur.elems, lane);
+                int32_t left = 0;
+                if (lane == 0) {
+                    sh.sum[i] = s;
+                    __threadfence_block();
+                    left = atomicSub(&sh.left[cur.batch], 1);
+                }
+                done = __shfl_sync(kFull, left, 0) == 1 ? cur.batch : -1;      // its last block
             }
-            int32_t done = __shfl_sync(kFull, left, 0) == 1 ? cur.batch : -1;      // its last block
             if (next >= blocks) {
                 __threadfence_block();
                 if (batch < 0) {
@@ -1236,15 +1308,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
                     done = -1;
                 }
                 while (batch >= 0) {
-                    int32_t u;
-                    double sumsq;
-                    const bool active = batch_sums(p, sh, batch, u, sumsq, lane);
-                    if (MODE == kStepPartials) {
-                        if (active)
-                            p.out_sumsq[u] = sumsq;
-                    } else {
-                        unit_epilogue(p, active, u, sumsq, alpha, beta, t);
-                    }
+                    run_batch(batch);
                     batch = done;
                     done = -1;
                 }
@@ -1283,7 +1347,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
                         pend_s = s;
                     }
                     if (++npend == 32) {
-                        unit_epilogue_call(p, true, pend_b, pend_s, alpha, beta, t);
+                        unit_epilogue_call<kDense>(p, true, pend_b, pend_s, alpha, beta, t);
                         npend = 0;
                     }
                 }
@@ -1342,7 +1406,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         }
         if (MODE == kStepFull) {
             if (npend > 0)
-                unit_epilogue_call(p, lane < npend, pend_b, pend_s, alpha, beta, t);
+                unit_epilogue_call<kDense>(p, lane < npend, pend_b, pend_s, alpha, beta, t);
         }
     }
     if (MODE == kStepPartials)
@@ -1359,7 +1423,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         s_misc[kMiscLast] = ticket_acq_rel(&p.ctl->ctas_done) == gridDim.x - 1 ? 1u : 0u;
     __syncthreads();
     if (s_misc[kMiscLast]) {
-        select_and_commit(p, s_t, s_hist, s_misc, s_red, s_keys);
+        select_and_commit<kDense>(p, s_t, s_hist, s_misc, s_red, s_keys);
     }
 }
 
@@ -1378,9 +1442,12 @@ cudaError_t launch_mode(const StepParams &p, int dtype, int num_ctas, cudaStream
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    constexpr bool kLists = MODE != kStepPartials;        // the partial sums come before either
     if (dtype == 1)
-        return cudaLaunchKernelEx(&cfg, gnmr_step_kernel<1, MODE, V>, p);
-    return cudaLaunchKernelEx(&cfg, gnmr_step_kernel<0, MODE, V>, p);
+        return cudaLaunchKernelEx(&cfg, kLists && !p.dense ? gnmr_step_kernel<1, MODE, V, false>
+                                                           : gnmr_step_kernel<1, MODE, V, kLists>, p);
+    return cudaLaunchKernelEx(&cfg, kLists && !p.dense ? gnmr_step_kernel<0, MODE, V, false>
+                                                       : gnmr_step_kernel<0, MODE, V, kLists>, p);
 }
 
 template <int V>
@@ -1408,30 +1475,35 @@ namespace {
 // The key cache is dynamic shared memory above the 48 KiB default, an opt-in
 // that is a per-device function attribute: set for every instance a handle
 // launches, on the current device.
-template <int DT, int V>
+template <int DT, int V, bool kDense>
 cudaError_t prepare_variant(int *ctas_per_sm)
 {
     const int bytes = static_cast<int>(kKeyCacheBytes);
-    cudaError_t e = cudaFuncSetAttribute(gnmr_step_kernel<DT, kStepFull, V>,
+    cudaError_t e = cudaFuncSetAttribute(gnmr_step_kernel<DT, kStepFull, V, kDense>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gnmr_step_kernel<0, kStepFinish, kVariantSmall>,
+        e = cudaFuncSetAttribute(gnmr_step_kernel<0, kStepFinish, kVariantSmall, kDense>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, gnmr_step_kernel<DT, kStepFull, V>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, gnmr_step_kernel<DT, kStepFull, V, kDense>,
                                                           kThreads, kKeyCacheBytes);
     return e;
 }
 
+template <int V>
+cudaError_t prepare(int dtype, bool dense, int *ctas_per_sm)
+{
+    if (dtype == 1)
+        return dense ? prepare_variant<1, V, true>(ctas_per_sm) : prepare_variant<1, V, false>(ctas_per_sm);
+    return dense ? prepare_variant<0, V, true>(ctas_per_sm) : prepare_variant<0, V, false>(ctas_per_sm);
+}
+
 }  // namespace
 
-cudaError_t step_occupancy(int dtype, int variant, int *ctas_per_sm)
+cudaError_t step_occupancy(int dtype, int variant, bool dense, int *ctas_per_sm)
 {
-    if (variant == kVariantBulk)
-        return dtype == 1 ? prepare_variant<1, kVariantBulk>(ctas_per_sm)
-                          : prepare_variant<0, kVariantBulk>(ctas_per_sm);
-    return dtype == 1 ? prepare_variant<1, kVariantSmall>(ctas_per_sm)
-                      : prepare_variant<0, kVariantSmall>(ctas_per_sm);
+    return variant == kVariantBulk ? prepare<kVariantBulk>(dtype, dense, ctas_per_sm)
+                                   : prepare<kVariantSmall>(dtype, dense, ctas_per_sm);
 }
 
 }  // namespace gnmr

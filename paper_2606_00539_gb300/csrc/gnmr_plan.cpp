@@ -39,7 +39,7 @@ struct Point {
 }  // namespace
 
 bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int32_t *seg_unit,
-                    int32_t num_units, int elem_bytes, int32_t max_runs, Plan &out)
+                    int32_t num_units, int elem_bytes, int32_t max_runs, Plan &out, const std::vector<int64_t> *targets)
 {
     if (num_segments < 1 || num_units < 1 || !seg_lengths || !seg_unit ||
         (elem_bytes != 2 && elem_bytes != 4) || max_runs < 1)
@@ -68,14 +68,14 @@ bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int3
     }
     const int64_t total = cstart[S];
     const int64_t want = (total + kMinRunBytes - 1) / kMinRunBytes;
-    const int64_t W = std::max<int64_t>(1, std::min<int64_t>(want, max_runs));
+    const int64_t W = targets ? int64_t(targets->size()) + 1 : std::max<int64_t>(1, std::min<int64_t>(want, max_runs));
     const int64_t align = std::max<int64_t>(1, kSplitBytes / elem_bytes);
 
     std::vector<Point> cuts;
     cuts.reserve(W + 1);
     cuts.push_back({0, 0});
     for (int64_t w = 1; w < W; ++w) {
-        const int64_t target = (int64_t)((__int128)total * w / W);
+        const int64_t target = targets ? (*targets)[w - 1] : (int64_t)((__int128)total * w / W);
         // segment g with cstart[g] <= target < cstart[g + 1]
         int64_t g = (int64_t)(std::upper_bound(cstart.begin(), cstart.end(), target) - cstart.begin()) - 1;
         g = std::min<int64_t>(std::max<int64_t>(g, 0), S - 1);
@@ -130,6 +130,32 @@ bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int3
     return true;
 }
 
+// Cost at which each run of a small arena ends, whole units wherever they are
+// at most kWholeUnitBytes: a run ends with the unit that takes it to `run`.
+static std::vector<int64_t> whole_unit_targets(int64_t num_segments, const int64_t *seg_lengths, const int32_t *seg_unit,
+                                               int elem_bytes, int64_t run)
+{
+    std::vector<int64_t> targets;
+    int64_t cost = 0, begin = 0;                             // of the stream so far; of the current run
+    for (int64_t g = 0; g < num_segments;) {
+        const int32_t u = seg_unit[g];
+        int64_t unit = kUnitCostBytes;
+        for (; g < num_segments && seg_unit[g] == u; ++g)
+            unit += std::max<int64_t>(seg_lengths[g], 1) * elem_bytes;
+        const int64_t pieces = (unit + kWholeUnitBytes - 1) / kWholeUnitBytes;
+        for (int64_t k = 1; k < pieces; ++k)
+            targets.push_back(cost + unit * k / pieces);
+        if (pieces > 1)
+            begin = targets.back();
+        cost += unit;
+        if (cost - begin >= run && g < num_segments) {
+            targets.push_back(cost);
+            begin = cost;
+        }
+    }
+    return targets;
+}
+
 // Blocks: the pieces of one segment that a CTA's warps take in turn.  The sums
 // of a CTA's blocks live in its shared memory, kBlocksPerCta of them at most:
 // larger blocks first, then more CTAs than are resident, make room.
@@ -147,10 +173,14 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
         cost += seg_lengths[g] * elem_bytes;
     }
     int64_t ctas = std::min<int64_t>(max_ctas, std::max<int64_t>(1, cost / kMinCtaBytes));
+    std::vector<int64_t> targets;
+    const bool whole = cost <= max_ctas * kSmallArenaCtaBytes;
+    if (whole)
+        targets = whole_unit_targets(num_segments, seg_lengths, seg_unit, elem_bytes, std::max(kMinCtaBytes, cost / max_ctas));
     const int64_t granule = kSplitBytes / elem_bytes;
     for (int64_t bytes = kMinBlockBytes;;) {
         if (ctas > INT32_MAX / 2 || !plan_partition(num_segments, seg_lengths, seg_unit, num_units, elem_bytes,
-                                                    static_cast<int32_t>(ctas), out))
+                                                    static_cast<int32_t>(ctas), out, whole ? &targets : nullptr))
             return false;
         blocks.cta.clear();
         blocks.block.clear();

@@ -758,14 +758,16 @@ def test_loop_shape_of_small_arenas(mib, extra, want, cuda_device):
 def _block_layout(name):
     if name == "block-edges":                             # around one and two blocks of 8 KiB
         return np.repeat([0, 1, 2047, 2048, 2049, 4095, 4096, 4097, 6145], 40)
+    if name == "whole-units":                             # around the 128 KiB up to which a small arena's stay whole
+        return np.array([1, 31_742, 31_743, 31_744, 31_745, 32_769, 0, 63_489, 63_487, 5, 100_003, 300] * 3)
     if name == "cta-spans":                               # units over two, three and more CTAs' parts
-        return np.array([5_000, 30_001, 12_000, 20_000, 7, 90_003, 1, 0, 50_000, 64_001])
+        return np.array([5_000, 300_001, 12_000, 20_000, 7, 990_003, 1, 0, 50_000, 64_001] * 8)
     if name == "more-than-resident":                      # more units than the resident CTAs' blocks
         return np.arange(700_001) % 4
     return np.array([70_000_001, 3, 0, 12_345])           # "one-giant": blocks larger than 8 KiB
 
 
-@pytest.mark.parametrize("name", ["block-edges", "cta-spans", "more-than-resident", "one-giant"])
+@pytest.mark.parametrize("name", ["block-edges", "whole-units", "cta-spans", "more-than-resident", "one-giant"])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_block_loop_layouts(name, dtype, cuda_device):
     """Norms of the small-unit loop at the edges of its plan, at odd offsets,
