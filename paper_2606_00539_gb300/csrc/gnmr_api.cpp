@@ -240,7 +240,7 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
     const bool large = c.loop_shape == GNMR_LOOP_AUTO
                            ? grad_bytes >= gnmr::kBulkArenaBytes && grad_bytes / c.num_units >= gnmr::kBulkUnitBytes
                            : c.loop_shape == GNMR_LOOP_LARGE_UNITS;
-    const int variant = large ? gnmr::kVariantBulk : gnmr::kVariantSmall;
+    int variant = large ? gnmr::kVariantBulk : gnmr::kVariantSmall;
     int sms = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
     if (e == cudaSuccess)
@@ -309,6 +309,15 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         } else {
             planned = gnmr::plan_blocks(S, seg_off.data(), seg_len.data(), seg_unit.data(), c.num_units, eb,
                                         sms * per_sm, plan, blocks);
+            if (blocks.grouped) {
+                variant = gnmr::kVariantGroups;
+                int groups_per_sm = 0;                 // (the grid may exceed it: no CTA waits for another)
+                e = gnmr::step_occupancy(c.dtype, variant, c.num_units <= gnmr::kDenseUnits, &groups_per_sm);
+                if (e != cudaSuccess) {
+                    delete h;
+                    return fail_create(GNMR_ERR_CUDA, format("device query failed: %s", cudaGetErrorString(e)));
+                }
+            }
         }
         if (!planned) {
             delete h;
@@ -418,7 +427,7 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         // small-unit loop: the warps that start on a block
         int64_t first_blocks = 0;
         for (const gnmr::CtaBlocks &b : blocks.cta)
-            first_blocks += std::min(b.count, gnmr::kWarpsPerCta);
+            first_blocks += std::min(b.turns, gnmr::kWarpsPerCta);
         const int32_t step_warps = static_cast<int32_t>(
             variant == gnmr::kVariantBulk ? std::min<int64_t>(plan.num_runs, grid_warps) : first_blocks);
         p.num_warps = step_warps;

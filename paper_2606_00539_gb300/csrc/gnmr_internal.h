@@ -14,13 +14,15 @@ namespace gnmr {
 // compiled variants of the streaming loop (gnmr_kernels.cu): kVariantSmall
 // (two resident CTAs per SM, each with a part of its own that its warps take
 // block by block) for layouts of small and mid-sized units and for small
-// arenas, kVariantBulk (one CTA per SM, deeper per-warp streams, runs
+// arenas (kVariantGroups: the same where short blocks dominate, several of them
+// to a warp at a time), kVariantBulk (one CTA per SM, deeper per-warp streams, runs
 // taken from a shared counter) for layouts whose mean unit holds at least
 // kBulkUnitBytes.
 constexpr int kThreads = 512;
 constexpr int kWarpsPerCta = kThreads / 32;
 constexpr int kVariantSmall = 0;
 constexpr int kVariantBulk = 1;
+constexpr int kVariantGroups = 2;
 constexpr int64_t kBulkUnitBytes = int64_t(1) << 20;
 // Below this many gradient bytes the large-unit loop's 64 KiB runs are too few
 // to balance: 168 units in 303 MB took 60.7 us with it, 57.9 with blocks; 84 in
@@ -67,19 +69,35 @@ constexpr int64_t kMaxBlockBytes = int64_t(1) << 20;
 constexpr int64_t kSmallArenaCtaBytes = int64_t(48) << 10;
 constexpr int64_t kWholeUnitBytes = int64_t(128) << 10;
 
-// A piece of one segment.
+// A piece of one segment.  `where`: its epilogue batch, counted from the CTA's
+// first unit (8 bits), the slot of its sum (12 bits: its place in the CTA's
+// blocks in unit order) and log2 of the lanes that stream it (3 bits).
 struct alignas(16) Block {
     int64_t start;    // first element, in the arena
-    int32_t elems;
-    int32_t batch;    // epilogue batch, counted from the CTA's first unit
+    int32_t elems;    // -1: no block
+    uint32_t where;
 };
+constexpr uint32_t kSlotShift = 8, kLanesShift = 20;
+static_assert(kBlocksPerCta / kBatch < (1 << kSlotShift) && kBlocksPerCta <= (1 << (kLanesShift - kSlotShift)), "Block::where");
+// What a warp takes at a time with kVariantGroups: up to kItemBlocks blocks of
+// one batch, each streamed by 32, 16, 8 or 4 lanes with kGroupVecs 16-byte
+// vectors a lane; kVariantSmall takes one block, streamed by the whole warp.
+// Planned where it makes at most kGroupedShare of the turns: a turn is about 2 us
+// of a warp, whatever its size, mostly the latency of its loads.  100,000 bf16
+// units of 55-440 elements 55.7 -> 34.2 us, of 64-512 fp32 elements 52.2 -> 36.6,
+// 30,000 of 48-4,096 bf16 elements 31.0 -> 28.1.
+constexpr int kItemBlocks = 8;
+constexpr int kGroupVecs = 8;
+constexpr double kGroupedShare = 0.75;
 struct alignas(16) CtaBlocks {
     int32_t first, count;         // blocks
     int32_t unit, units;          // first unit touched, and how many
+    int32_t turn, turns;          // what the warps take: entries of `block`, in kItemBlocks with kVariantGroups
     // the first and the last unit (one and the same if units == 1), which
     // other CTAs may have parts of: number of parts (1: none), the unit's
     // first partial slot, and this CTA's slot from there
     int32_t parts[2], slot[2];
+    int32_t pad[2];
     int64_t base[2];
 };
 
@@ -164,7 +182,7 @@ struct StepParams {
     const int64_t *run_seg;      // [R + 1] first segment of each run
     const int64_t *run_pos;      // [R + 1]
     const CtaBlocks *cta_blocks; // [num_ctas] small-unit loop: each CTA's part,
-    const Block *block;          // the blocks of all CTAs
+    const Block *block;          // the blocks of all CTAs, in the order the warps take them
     const int32_t *unit_block;   // [U + 1] and the first block of each unit
     const int32_t *first_run;    // [U] first run (small-unit loop: CTA) touching unit b
     const int32_t *num_parts;    // [U]
@@ -242,8 +260,9 @@ bool plan_partition(int64_t num_segments, const int64_t *seg_lengths, const int3
 // The blocks of a plan with one run per CTA (small-unit loop).
 struct BlockPlan {
     std::vector<CtaBlocks> cta;       // [num_runs]
-    std::vector<Block> block;
+    std::vector<Block> block;         // kItemBlocks entries a turn if grouped
     std::vector<int32_t> unit_block;  // [U + 1]
+    bool grouped = false;
 };
 
 // Cuts the stream into one run per CTA (about max_ctas of them, more where a

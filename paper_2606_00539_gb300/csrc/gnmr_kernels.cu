@@ -79,11 +79,19 @@ template <> struct Shape<kVariantSmall> {
     static constexpr int kUnroll = 8;
     static constexpr int kMinCtas = 2;
     static constexpr bool kBlocks = true;             // blocks of the CTA's own part, in turn
+    static constexpr bool kGroups = false;
+};
+template <> struct Shape<kVariantGroups> {
+    static constexpr int kUnroll = 8;
+    static constexpr int kMinCtas = 2;
+    static constexpr bool kBlocks = true;
+    static constexpr bool kGroups = true;             // several short blocks a turn
 };
 template <> struct Shape<kVariantBulk> {
     static constexpr int kUnroll = 16;
     static constexpr int kMinCtas = 1;
     static constexpr bool kBlocks = false;            // runs taken from a global counter
+    static constexpr bool kGroups = false;
 };
 
 __device__ __forceinline__ double pick_threshold(double override_value, int64_t t, int64_t warmup,
@@ -1167,6 +1175,14 @@ __device__ __forceinline__ bool batch_sums(const StepParams &p, const BlockShare
     return active;
 }
 
+// The lane's entry of a turn (large blocks: the one entry, in every lane).
+template <int V>
+__device__ __forceinline__ Block turn_entry(const StepParams &p, int32_t turn, int lane)
+{
+    return Shape<V>::kGroups ? p.block[static_cast<int64_t>(turn) * kItemBlocks + lane / (32 / kItemBlocks)]
+                             : p.block[turn];
+}
+
 // MODE kStepFull: the whole step.  kStepPartials: phase 1 only, each unit's
 // sum of squares written to out_sumsq (the first half of a sharded step).
 // kStepFinish: no gradient read; phases 2-3 on the sums in in_sumsq (the
@@ -1185,14 +1201,15 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
     const int lane = threadIdx.x & 31;
     const int warp = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
     BlockShared &sh = *reinterpret_cast<BlockShared *>(s_keys);
-    int32_t first_block = 0, blocks = 0;
+    int32_t first_turn = 0, turns = 0;
     Block cur{};
     if (MODE != kStepFinish && Shape<V>::kBlocks) {
         // The plan never changes after create: read while the kernel before
         // this one on the stream is still running.
         const CtaBlocks &plan = p.cta_blocks[blockIdx.x];
-        first_block = plan.first;
-        blocks = plan.count;
+        const int32_t first_block = plan.first, blocks = plan.count;
+        first_turn = plan.turn;
+        turns = plan.turns;
         const int32_t unit = plan.unit, units = plan.units;
         for (int32_t k = threadIdx.x; k < units; k += kThreads) {
             const int32_t end = p.unit_block[unit + k + 1] - first_block;
@@ -1210,8 +1227,8 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             sh.cta = plan;
         }
         const int32_t i = threadIdx.x >> 5;
-        if (i < blocks)
-            cur = p.block[first_block + i];
+        if (i < turns)
+            cur = turn_entry<V>(p, first_turn + i, lane);
         __syncthreads();
     }
     // Launched as a programmatic dependent of whatever precedes it on the
@@ -1277,31 +1294,55 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             if (__shfl_sync(kFull, left, 0) == 1)        // every block was summed before
                 batch = last_batch;
         }
-        while (i < blocks || (kDense && batch >= 0)) {
-            int32_t next = blocks, done = -1;
+        while (i < turns || (kDense && batch >= 0)) {
+            int32_t next = turns, done = -1;
             Block follow = cur;
-            if (!kDense || i < blocks) {
+            if (!kDense || i < turns) {
                 // the next block's index and table entry travel under this one's stream
                 if (batch < 0) {
                     if (lane == 0)
                         next = atomicAdd(&sh.next, 1);
                     next = __shfl_sync(kFull, next, 0);
                 }
-                follow = p.block[first_block + (next < blocks ? next : i)];
+                follow = turn_entry<V>(p, first_turn + (next < turns ? next : i), lane);
+                const int log2 = static_cast<int>(__shfl_sync(kFull, cur.where, 0) >> kLanesShift);
+                if (Shape<V>::kGroups) {
+                    // the entry of the lane's group (entry j travels in lanes 4 j ...)
+                    const int from = (lane >> log2) * (32 / kItemBlocks);
+                    cur.start = __shfl_sync(kFull, cur.start, from);
+                    cur.elems = __shfl_sync(kFull, cur.elems, from);
+                    cur.where = __shfl_sync(kFull, cur.where, from);
+                }
                 const char *seg = arena + cur.start * kEB;
                 bool suspect;
-                double s = warp_segment_sumsq<DT, Shape<V>::kUnroll>(seg, cur.elems, lane, suspect);
-                if (suspect)
-                    s = warp_segment_sumsq_f64<DT>(seg, cur.elems, lane);
-                int32_t left = 0;
-                if (lane == 0) {
-                    sh.sum[i] = s;
-                    __threadfence_block();
-                    left = atomicSub(&sh.left[cur.batch], 1);
+                double s;
+                if (!Shape<V>::kGroups || log2 == 5) {
+                    s = warp_segment_sumsq<DT, Shape<V>::kUnroll>(seg, cur.elems, lane, suspect);
+                    if (suspect)
+                        s = warp_segment_sumsq_f64<DT>(seg, cur.elems, lane);
+                } else {
+                    s = group_segment_sumsq<DT, kGroupVecs>(seg, max(cur.elems, 0), 1 << log2, lane, suspect);
+                    for (unsigned m = __ballot_sync(kFull, suspect); m;) {         // one group at a time
+                        const int l = __ffs(m) - 1;
+                        const double x = warp_segment_sumsq_f64<DT>(
+                            arena + __shfl_sync(kFull, cur.start, l) * kEB, __shfl_sync(kFull, cur.elems, l), lane);
+                        if (lane >> log2 == l >> log2)
+                            s = x;
+                        m &= ~(((1u << (1 << log2)) - 1u) << l);
+                    }
                 }
-                done = __shfl_sync(kFull, left, 0) == 1 ? cur.batch : -1;      // its last block
+                const uint32_t in = cur.where % (1u << kSlotShift);
+                int32_t left = 0;
+                if ((lane & ((1 << log2) - 1)) == 0 && (!Shape<V>::kGroups || cur.elems >= 0)) {
+                    sh.sum[(cur.where >> kSlotShift) % (1u << (kLanesShift - kSlotShift))] = s;
+                    __threadfence_block();
+                    left = atomicSub(&sh.left[in], 1);
+                }
+                // its batch's last block (a turn's blocks are all of one batch)
+                if (Shape<V>::kGroups ? __any_sync(kFull, left == 1) : __shfl_sync(kFull, left, 0) == 1)
+                    done = static_cast<int32_t>(__shfl_sync(kFull, in, 0));
             }
-            if (next >= blocks) {
+            if (next >= turns) {
                 __threadfence_block();
                 if (batch < 0) {
                     batch = done;
@@ -1315,8 +1356,8 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
                 if (lane == 0)
                     next = atomicAdd(&sh.next, 1);
                 next = __shfl_sync(kFull, next, 0);
-                if (next < blocks)
-                    cur = p.block[first_block + next];
+                if (next < turns)
+                    cur = turn_entry<V>(p, first_turn + next, lane);
             } else {
                 batch = done;
                 cur = follow;
@@ -1467,6 +1508,8 @@ cudaError_t launch_step(const StepParams &p, int dtype, int num_ctas, cudaStream
         return launch_mode<kStepFinish, kVariantSmall>(p, 0, num_ctas, stream);
     if (variant == kVariantBulk)
         return launch_variant<kVariantBulk>(p, dtype, num_ctas, stream, mode);
+    if (variant == kVariantGroups)
+        return launch_variant<kVariantGroups>(p, dtype, num_ctas, stream, mode);
     return launch_variant<kVariantSmall>(p, dtype, num_ctas, stream, mode);
 }
 
@@ -1502,8 +1545,9 @@ cudaError_t prepare(int dtype, bool dense, int *ctas_per_sm)
 
 cudaError_t step_occupancy(int dtype, int variant, bool dense, int *ctas_per_sm)
 {
-    return variant == kVariantBulk ? prepare<kVariantBulk>(dtype, dense, ctas_per_sm)
-                                   : prepare<kVariantSmall>(dtype, dense, ctas_per_sm);
+    return variant == kVariantBulk     ? prepare<kVariantBulk>(dtype, dense, ctas_per_sm)
+           : variant == kVariantGroups ? prepare<kVariantGroups>(dtype, dense, ctas_per_sm)
+                                       : prepare<kVariantSmall>(dtype, dense, ctas_per_sm);
 }
 
 }  // namespace gnmr

@@ -156,6 +156,59 @@ static std::vector<int64_t> whole_unit_targets(int64_t num_segments, const int64
     return targets;
 }
 
+// Packs the blocks of each CTA into turns of several short ones, if that saves
+// enough turns.  A turn holds blocks of one batch: the longest not yet taken
+// sets the lanes per block, and the next longest fill the rest of the warp.
+static void group_blocks(BlockPlan &plan, int elem_bytes)
+{
+    const auto log2_lanes = [&](int32_t elems) {
+        int l = 2;
+        while (l < 5 && int64_t(elems) * elem_bytes > (int64_t(16) * kGroupVecs << l))
+            ++l;
+        return l;
+    };
+    if (plan.block.size() <= 2 * kWarpsPerCta * plan.cta.size())
+        return;                                           // at most two turns a warp as it is
+    int64_t lanes = 0;                                    // if every turn were full
+    for (const Block &b : plan.block)
+        lanes += int64_t(1) << log2_lanes(b.elems);
+    if (lanes > 32 * kGroupedShare * plan.block.size())
+        return;
+    std::vector<Block> turns;
+    std::vector<CtaBlocks> cta = plan.cta;
+    turns.reserve(static_cast<size_t>(kGroupedShare * plan.block.size()) * kItemBlocks);
+    std::vector<Block> batch;
+    for (CtaBlocks &c : cta) {
+        c.turn = static_cast<int32_t>(turns.size() / kItemBlocks);
+        for (int32_t i = 0; i < c.count;) {
+            batch.clear();
+            const uint32_t k = plan.block[c.first + i].where % (1u << kSlotShift);
+            for (; i < c.count && plan.block[c.first + i].where % (1u << kSlotShift) == k; ++i)
+                batch.push_back(plan.block[c.first + i]);
+            // (equal lengths in the order of their slots: the plan is a function of the layout)
+            std::sort(batch.begin(), batch.end(), [](const Block &x, const Block &y) {
+                return x.elems != y.elems ? x.elems > y.elems : x.where < y.where;
+            });
+            for (size_t j = 0; j < batch.size();) {
+                const int l = log2_lanes(batch[j].elems);
+                const size_t n = std::min<size_t>(batch.size() - j, size_t(32) >> l);
+                for (size_t m = 0; m < size_t(kItemBlocks); ++m) {
+                    Block b = m < n ? batch[j + m] : Block{0, -1, 0};
+                    b.where = b.where % (1u << kLanesShift) | static_cast<uint32_t>(l) << kLanesShift;
+                    turns.push_back(b);
+                }
+                j += n;
+            }
+        }
+        c.turns = static_cast<int32_t>(turns.size() / kItemBlocks) - c.turn;
+    }
+    if (turns.size() / kItemBlocks > kGroupedShare * plan.block.size() || turns.size() > size_t(INT32_MAX / 2))
+        return;
+    plan.cta = std::move(cta);
+    plan.block = std::move(turns);
+    plan.grouped = true;
+}
+
 // Blocks: the pieces of one segment that a CTA's warps take in turn.  The sums
 // of a CTA's blocks live in its shared memory, kBlocksPerCta of them at most:
 // larger blocks first, then more CTAs than are resident, make room.
@@ -184,6 +237,8 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
             return false;
         blocks.cta.clear();
         blocks.block.clear();
+        blocks.block.reserve(static_cast<size_t>(std::min(num_segments + cost / bytes + out.num_runs,
+                                                          int64_t(kBlocksPerCta) * out.num_runs)));
         blocks.unit_block.assign(num_units + 1, 0);
         bool fits = true;
         int32_t prev_unit = -1;
@@ -201,12 +256,15 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
                     blocks.unit_block[u] = static_cast<int32_t>(blocks.block.size());
                 prev_unit = u;
                 // equal pieces of whole granules; an empty segment is one empty piece
-                const int64_t pieces = std::max<int64_t>(1, (n * elem_bytes + bytes - 1) / bytes);
-                const int64_t per = ((n + pieces - 1) / pieces + granule - 1) / granule * granule;
+                const int64_t pieces = n * elem_bytes <= bytes ? 1 : (n * elem_bytes + bytes - 1) / bytes;
+                const int64_t per = pieces == 1 ? n : ((n + pieces - 1) / pieces + granule - 1) / granule * granule;
                 int64_t at = 0;
                 do {
                     const int64_t m = std::min(std::max<int64_t>(per, 1), n - at);
-                    blocks.block.push_back({seg_offsets[g] + pos + at, static_cast<int32_t>(m), (u - c.unit) / kBatch});
+                    const uint32_t slot = static_cast<uint32_t>(blocks.block.size() - c.first) % (1u << (kLanesShift - kSlotShift));
+                    blocks.block.push_back({seg_offsets[g] + pos + at, static_cast<int32_t>(m),
+                                            static_cast<uint32_t>((u - c.unit) / kBatch) % (1u << kSlotShift) |
+                                                slot << kSlotShift | 5u << kLanesShift});
                     at += m;
                 } while (at < n);
                 c.units = u - c.unit + 1;
@@ -216,6 +274,8 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
                 }
             }
             c.count = static_cast<int32_t>(blocks.block.size()) - c.first;
+            c.turn = c.first;
+            c.turns = c.count;
             for (int e = 0; e < 2; ++e) {
                 const int32_t u = e == 0 ? c.unit : c.unit + c.units - 1;
                 c.parts[e] = out.num_parts[u];
@@ -226,6 +286,7 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
         }
         if (fits) {
             blocks.unit_block[num_units] = static_cast<int32_t>(blocks.block.size());
+            group_blocks(blocks, elem_bytes);
             return true;
         }
         if (bytes < kMaxBlockBytes)

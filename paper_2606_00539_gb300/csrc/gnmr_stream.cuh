@@ -244,6 +244,79 @@ __device__ __forceinline__ double warp_segment_sumsq(const char *seg, int64_t n,
     return acc;
 }
 
+// Sums of squares of several short segments at once: the lanes in groups of
+// `lanes` (4, 8 or 16), each streaming n elements at seg with at most kVecs
+// vectors a lane.  Returns the group's sum in every lane of it and sets
+// `suspect` as warp_segment_sumsq() does, by group.  Called by all 32 lanes.
+template <int DT, int kVecs>
+__device__ __forceinline__ double group_segment_sumsq(const char *seg, int32_t n, int lanes, int lane, bool &suspect)
+{
+    constexpr int kEB = Elem<DT>::kBytes;
+    constexpr int kVE = kVecBytes / kEB;
+    const int gl = lane & (lanes - 1);
+    const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(seg)) & (kVecBytes - 1);
+    const int32_t head = min(static_cast<int32_t>(((kVecBytes - mis) & (kVecBytes - 1)) / kEB), n);
+    const int32_t nvec = (n - head) / kVE;
+    const int32_t tail_at = head + nvec * kVE;
+
+    const Vec *v = reinterpret_cast<const Vec *>(seg + head * kEB);
+    Vec r[kVecs];
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j)
+        r[j] = gl + lanes * j < nvec ? ld_stream(v + gl + lanes * j) : zero_vec();
+    uint32_t bits = 0;
+    float edge = 0.f;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {                          // up to 7 head and tail elements, 4 lanes at least
+        if (k == 1 && lanes >= kVE)
+            break;
+        const int32_t at = gl + lanes * k;
+        if (at < head) {
+            const uint32_t w = ld_elem_bits<DT>(seg + at * kEB);
+            bits |= w;
+            edge = fmaf(__uint_as_float(w), __uint_as_float(w), edge);
+        }
+        if (tail_at + at < n) {
+            const uint32_t w = ld_elem_bits<DT>(seg + (tail_at + at) * kEB);
+            bits |= w;
+            edge = fmaf(__uint_as_float(w), __uint_as_float(w), edge);
+        }
+    }
+    float a[kVecs];
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j) {
+        a[j] = vec_sumsq<DT>(r[j]);
+        bits |= vec_or(r[j]);
+    }
+#pragma unroll
+    for (int w = kVecs / 2; w > 0; w >>= 1)               // pairwise tree
+#pragma unroll
+        for (int j = 0; j < w; ++j)
+            a[j] += a[j + w];
+    const uint32_t tot = __float_as_uint(a[0] + edge);
+    uint32_t e = tot;
+    for (int o = lanes / 2; o > 0; o >>= 1)
+        e = max(e, __shfl_xor_sync(kFull, e, o));
+    e >>= 23;                                             // > 254 for NaN and Inf
+    const bool ok = e - 27u < 200u;
+    suspect = false;
+    if (__any_sync(kFull, !ok)) {
+        for (int o = lanes / 2; o > 0; o >>= 1)
+            bits |= __shfl_xor_sync(kFull, bits, o);
+        suspect = !ok && (bits & Elem<DT>::kMagnitude) != 0u;
+    }
+    // in fixed point, as in warp_segment_sumsq()
+    const uint32_t own = tot >> 23;
+    const uint32_t sh = min(e - own, 27u);
+    const uint32_t frac = own ? ((tot & 0x7fffffu) | 0x800000u) << 2 : 0u;
+    uint32_t sum = (frac + ((1u << sh) >> 1)) >> sh;
+    for (int o = lanes / 2; o > 0; o >>= 1)
+        sum += __shfl_xor_sync(kFull, sum, o);
+    const uint32_t lz = ok ? __clz(sum) : 0u;
+    const uint32_t m = sum << (lz + 1);
+    return ok ? __hiloint2double(static_cast<int>(((902u + e - lz) << 20) | (m >> 12)), static_cast<int>(m << 20)) : 0.0;
+}
+
 // Exact-product fallback: each element squared in fp64 (exact for fp32 and
 // bf16 inputs) and summed in fp64.  Taken only for segments flagged suspect.
 template <int DT>

@@ -814,3 +814,37 @@ def test_lane_totals_of_any_size(power, shape, cuda_device):
         # of non-negative terms, and 2^-26 of the largest lane 32 times; the root
         # halves it: 27 / 2 * 2^-24 + 16 * 2^-26 < 1.1e-6
         np.testing.assert_allclose(got, want, rtol=1.1e-6, atol=0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("start", [0, 1, 3])
+def test_short_units_share_a_warp(dtype, start, cuda_device):
+    """20,000 units at the edges of what 4, 8, 16 and 32 lanes stream, packed
+    without padding, some of zeros, some whose fp32 squares underflow or
+    overflow, some with a NaN or an Inf."""
+    import torch
+    eb = 4 if dtype == "f32" else 2
+    sizes = [b // eb + d for b in (16, 128, 512, 1024, 2048, 4096) for d in (-1, 0, 1)] + [0, 1, 2, 9]
+    rng = np.random.default_rng(start)
+    U = 20_000
+    lengths = rng.choice(np.array(sizes, np.int64), U)
+    offsets = start + np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64)
+    scale = rng.choice([1.0, 1.0, 1.0, 1e-3, 0.0, 1e-25, 1e25], U)
+    n = int(offsets[-1] + lengths[-1])
+    ids = torch.repeat_interleave(torch.arange(U, device=cuda_device), torch.from_numpy(lengths).to(cuda_device))
+    g = torch.Generator(cuda_device).manual_seed(start)
+    x = torch.zeros(n, dtype=torch.float64, device=cuda_device)
+    x[start:] = torch.randn(n - start, device=cuda_device, generator=g, dtype=torch.float64) * torch.from_numpy(scale).to(cuda_device)[ids]
+    for u, bad in ((77, float("nan")), (78, float("inf")), (4001, float("-inf"))):
+        if lengths[u]:
+            x[int(offsets[u] + lengths[u] // 2)] = bad
+    arena = x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    want = torch.zeros(U, dtype=torch.float64, device=cuda_device).index_add_(0, ids, arena[start:].double().square()).sqrt()
+    with Monitor(offsets, lengths, dtype=dtype, window=2) as mon:
+        stats = mon.new_stats()
+        mon.step(arena, stats=stats)
+        # at most 64 fp32 roundings per lane of non-negative terms, mostly of partial
+        # sums far below the total, and 2^-26 per lane; measured below 1e-7
+        torch.testing.assert_close(stats["norm"], want, rtol=1e-6, atol=0, equal_nan=True)
+        sums = mon.step_partials(arena)
+        assert torch.equal(sums.sqrt().nan_to_num(7.0), stats["norm"].nan_to_num(7.0))
