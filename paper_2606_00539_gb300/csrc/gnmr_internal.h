@@ -63,6 +63,13 @@ constexpr int kBlocksPerCta = 2048;
 constexpr int64_t kMinCtaBytes = int64_t(24) << 10;
 constexpr int64_t kMinBlockBytes = int64_t(8) << 10;
 constexpr int64_t kMaxBlockBytes = int64_t(1) << 20;
+// Layouts of units of kEvenUnitBytes and more on average: a CTA's part divided
+// by its warps, in as many equal rounds as keep a block within kEvenBlockBytes
+// or a little above (560 units of 224 KB, 26 KB a warp: one 26 KB round 27.5 us,
+// two of 13 KB 27.8, 8 KiB blocks 29.3, 24 KB blocks, 18 to a CTA, 31.3; a rank's
+// 303 MB of 168 units 56.9 -> 55.3; 84 units in 95 MB 36.6 -> 35.0).
+constexpr int64_t kEvenUnitBytes = int64_t(128) << 10;
+constexpr int64_t kEvenBlockBytes = int64_t(16) << 10;
 // Arenas of at most kSmallArenaCtaBytes of cost per resident CTA are cut between
 // units: joining the parts of a split unit takes longer than streaming a unit of
 // up to kWholeUnitBytes, 8 KiB a warp (64 units in 3.7 MB: 11.4 -> 10.1 us).

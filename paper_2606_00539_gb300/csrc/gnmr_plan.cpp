@@ -231,7 +231,11 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
     if (whole)
         targets = whole_unit_targets(num_segments, seg_lengths, seg_unit, elem_bytes, std::max(kMinCtaBytes, cost / max_ctas));
     const int64_t granule = kSplitBytes / elem_bytes;
-    for (int64_t bytes = kMinBlockBytes;;) {
+    // Few long units per CTA: blocks that make whole turns of its warps.
+    const int64_t share = cost / ctas / kWarpsPerCta;
+    const bool even = !whole && cost / num_units >= kEvenUnitBytes && share >= kMinBlockBytes;
+    const int64_t rounds = (share + kEvenBlockBytes - 1) / kEvenBlockBytes;
+    for (int64_t bytes = even ? (share + rounds - 1) / rounds : kMinBlockBytes;;) {
         if (ctas > INT32_MAX / 2 || !plan_partition(num_segments, seg_lengths, seg_unit, num_units, elem_bytes,
                                                     static_cast<int32_t>(ctas), out, whole ? &targets : nullptr))
             return false;
@@ -256,7 +260,7 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
                     blocks.unit_block[u] = static_cast<int32_t>(blocks.block.size());
                 prev_unit = u;
                 // equal pieces of whole granules; an empty segment is one empty piece
-                const int64_t pieces = n * elem_bytes <= bytes ? 1 : (n * elem_bytes + bytes - 1) / bytes;
+                const int64_t pieces = n * elem_bytes <= bytes ? 1 : (n * elem_bytes + (even ? bytes / 2 : bytes - 1)) / bytes;
                 const int64_t per = pieces == 1 ? n : ((n + pieces - 1) / pieces + granule - 1) / granule * granule;
                 int64_t at = 0;
                 do {
