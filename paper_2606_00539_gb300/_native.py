@@ -246,9 +246,11 @@ def gnmr_actuator_create(offsets, rows, cols, dtype: int, device: int = 0) -> in
 
 def gnmr_actuator_apply(handle: int, d_in: int, d_out: int, arena_elems: int, d_mask,
                         lowcost_format: int, recovery_format: int, stream: int = 0) -> None:
-    st = load().gnmr_actuator_apply(handle, d_in, d_out, int(arena_elems), d_mask,
-                                    int(lowcost_format), int(recovery_format), stream)
-    _check(st, None)
+    lib = _lib if _lib is not None else load()
+    st = lib.gnmr_actuator_apply(handle, d_in, d_out, int(arena_elems), d_mask,
+                                 int(lowcost_format), int(recovery_format), stream)
+    if st != GNMR_OK:
+        _check(st, None)
 
 
 def gnmr_actuator_destroy(handle: int) -> None:

@@ -762,15 +762,17 @@ gnmr_status gnmr_actuator_apply(gnmr_actuator *a, const void *d_in, void *d_out,
         return act_fail(GNMR_ERR_LAYOUT, "actuator: buffer shorter than the layout");
     if (a->tiles == 0)
         return GNMR_OK;
-    int prev = 0;
+    int prev = a->device;
     cudaGetDevice(&prev);
-    cudaSetDevice(a->device);
+    if (prev != a->device)                        // switching costs as much as a tenth of a small launch
+        cudaSetDevice(a->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const cudaError_t e = a->dtype == GNMR_DTYPE_BF16 ? launch<1>(*a, d_in, d_out, d_mask, low, rec, st)
                                                       : launch<0>(*a, d_in, d_out, d_mask, low, rec, st);
     if (e != cudaSuccess)
         cudaGetLastError();                       // reported here, not by the caller's next call
-    cudaSetDevice(prev);
+    if (prev != a->device)
+        cudaSetDevice(prev);
     if (e != cudaSuccess)
         return act_fail(GNMR_ERR_CUDA, std::string("actuator launch: ") + cudaGetErrorString(e));
     return GNMR_OK;
