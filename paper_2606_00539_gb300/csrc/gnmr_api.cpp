@@ -434,13 +434,14 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         p.num_runs = plan.num_runs;
         p.dense = U <= gnmr::kDenseUnits ? 1 : 0;
         p.window = c.window;
+        p.window_length = gnmr::make_divisor(c.window);
         p.max_o = c.max_o;
         p.lock_len = c.lock_len;
         p.warmup_steps = c.warmup_steps;
-        p.alpha_init = c.alpha_init;
-        p.alpha_main = c.alpha_main;
-        p.beta_init = c.beta_init;
-        p.beta_main = c.beta_main;
+        p.alpha_init = gnmr::make_divisor(c.alpha_init);
+        p.alpha_main = gnmr::make_divisor(c.alpha_main);
+        p.beta_init = gnmr::make_divisor(c.beta_init);
+        p.beta_main = gnmr::make_divisor(c.beta_main);
         p.eps = c.eps;
 
         h->cfg = c;
@@ -508,8 +509,8 @@ gnmr_status gnmr_step(gnmr_handle *h, const void *d_arena, int64_t arena_elems, 
         p.out_counts = stats->counts;
         p.out_delta_mem = stats->delta_mem;
     }
-    p.alpha_override = h->alpha_override;
-    p.beta_override = h->beta_override;
+    p.alpha_override = gnmr::make_divisor(h->alpha_override);
+    p.beta_override = gnmr::make_divisor(h->beta_override);
     const cudaError_t e = gnmr::launch_step(p, h->cfg.dtype, h->num_ctas, static_cast<cudaStream_t>(stream),
                                             gnmr::kStepFull, h->variant);
     if (e != cudaSuccess) {
@@ -578,8 +579,8 @@ gnmr_status gnmr_finish(gnmr_handle *h, const double *d_sumsq, void *stream, uin
         p.out_counts = stats->counts;
         p.out_delta_mem = stats->delta_mem;
     }
-    p.alpha_override = h->alpha_override;
-    p.beta_override = h->beta_override;
+    p.alpha_override = gnmr::make_divisor(h->alpha_override);
+    p.beta_override = gnmr::make_divisor(h->beta_override);
     const cudaError_t e = gnmr::launch_step(p, h->cfg.dtype, h->finish_ctas, static_cast<cudaStream_t>(stream),
                                             gnmr::kStepFinish);
     if (e != cudaSuccess) {

@@ -180,6 +180,17 @@ struct StateHeader {
     int64_t reserved;
 };
 
+// A divisor fixed for many divisions, with its reciprocal rounded to nearest; 0
+// where the device has to divide (see divide_by).
+struct Divisor {
+    double value;
+    double inverse;
+};
+inline Divisor make_divisor(double v)
+{
+    return {v, v >= 0x1p-200 && v <= 0x1p+200 ? 1.0 / v : 0.0};
+}
+
 struct StepParams {
     const void *arena;
     const int64_t *offset;       // [S] segment offsets, segments grouped by unit
@@ -224,8 +235,10 @@ struct StepParams {
     int32_t dense;               // 1: at most kDenseUnits units, selected from one entry each
     int32_t num_runs;            // R; runs num_warps .. R - 1 are taken dynamically
     int64_t warmup_steps;
-    double alpha_init, alpha_main, beta_init, beta_main, eps;
-    double alpha_override, beta_override;  // NaN = two-stage schedule
+    Divisor alpha_init, alpha_main, beta_init, beta_main;
+    Divisor alpha_override, beta_override;  // NaN = two-stage schedule
+    Divisor window_length;
+    double eps;
 };
 
 // Step kernel modes: the full step, its gradient half (per-unit sums of

@@ -282,3 +282,31 @@ def test_selection_of_few_units(units, kind, cuda_device, monkeypatch):
     _drive(steps)
     _drive(steps, policy=1)
     _drive(steps, policy=2, static_warmup_steps=2, static_fraction=0.3)
+
+
+@pytest.mark.parametrize("alpha,beta,window", [(1.1, 1.3, 5), (0.9, 7.0 / 3.0, 3), (1.5, 1.1, 8), (1.0000000000000002, 1e-3, 13),
+                                               (2.0 ** 200, 2.0 ** -200, 7), (1e61, 1e-61, 1), (1.9999999999999998, 3.0, 6)])
+def test_threshold_and_window_divisions_round_correctly(alpha, beta, window, cuda_device):
+    """GNMR / alpha, Delta / beta and the window's mean are divided through
+    reciprocals: risks over 300 orders of magnitude (zeros and infinities
+    among them) equal the oracle's bit for bit, one lane and four lanes a unit."""
+    import torch
+    for units in (20_000, 500):
+        rng = np.random.default_rng(units + window)
+        kw = dict(window=window, max_o=5, lock_len=1, eps=0.0)
+        mon = Monitor(np.zeros(units, np.int64), np.zeros(units, np.int64), dtype="f32", alpha=alpha, beta=beta, **kw)
+        ctl = oracle.Controller(units, alpha=(alpha, alpha), beta=(beta, beta), **kw)
+        stats = mon.new_stats()
+        try:
+            for t in range(window + 4):
+                n = np.exp(rng.uniform(-1.0, 1.0, units) if t <= window else rng.uniform(-345.0, 345.0, units))
+                if t > 1:
+                    n[rng.random(units) < 0.05] = 0.0
+                sums = n * n
+                mon.finish(torch.from_numpy(sums).to(cuda_device), stats=stats)
+                want = ctl.step(np.sqrt(sums))
+                got = stats["risk"].cpu().numpy()
+                assert np.array_equal(got.view(np.uint64), want.risk.view(np.uint64)), f"step {t + 1}"
+        finally:
+            mon.close()
+            ctl.close()
