@@ -1147,7 +1147,8 @@ struct BlockShared {
     Preload pre;                                  // of the CTA's last batch
     CtaBlocks cta;
     int32_t left[kBlocksPerCta / kBatch + 2];     // blocks of each batch not yet summed
-    int32_t next;                                 // next block to hand out
+    uint32_t ready[2];                            // batches that wait for a warp, by bit
+    int32_t next;                                 // next turn to hand out
 };
 
 // The sums of a batch's units, one per lane (lane j: unit0 + j), from their
@@ -1195,6 +1196,33 @@ __device__ __forceinline__ bool batch_sums(const StepParams &p, const BlockShare
         }
     }
     return active;
+}
+
+// Leaves a batch whose blocks are all summed for the next warp without a turn.
+__device__ __forceinline__ void leave_batch(BlockShared &sh, int32_t batch, int lane)
+{
+    if (lane == 0) {
+        __threadfence_block();
+        atomicOr(&sh.ready[batch / 32], 1u << (batch % 32));
+    }
+}
+// Takes one of the batches left, or returns -1.
+__device__ __forceinline__ int32_t take_batch(BlockShared &sh, int lane)
+{
+    int32_t batch = -1;
+    if (lane == 0) {
+        for (int w = 0; w < 2 && batch < 0; ++w) {
+            uint32_t m = *const_cast<volatile uint32_t *>(&sh.ready[w]);
+            while (m != 0 && batch < 0) {
+                const uint32_t bit = m & (0u - m);
+                m = atomicAnd(&sh.ready[w], ~bit);         // what was there before
+                if (m & bit)
+                    batch = 32 * w + __ffs(bit) - 1;
+            }
+        }
+        __threadfence_block();
+    }
+    return __shfl_sync(kFull, batch, 0);
 }
 
 // The lane's entry of a turn (large blocks: the one entry, in every lane).
@@ -1246,6 +1274,7 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         }
         if (threadIdx.x == 0) {
             sh.next = kWarpsPerCta;
+            sh.ready[0] = sh.ready[1] = 0;
             sh.cta = plan;
         }
         const int32_t i = threadIdx.x >> 5;
@@ -1275,8 +1304,12 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
         // t, alpha_t and beta_t are fixed for the whole step.
         const int64_t t = MODE == kStepFull ? __ldcg(&p.ctl->steps) + 1 : 0;
         const char *arena = static_cast<const char *>(p.arena);
-        // A warp that completes a batch runs it only when it has no block in
-        // hand: a block kept waiting for an epilogue would hold up its own batch.
+        // A warp that completes a batch runs it only when it has no turn in hand: a
+        // block kept waiting for an epilogue would hold up its own batch.  With many
+        // units any warp without a turn can take it till then, and the second one
+        // that the warp may complete with that turn: with both run by the one warp,
+        // one after the other, the CTAs of 30,000 short units ended after 17.5 us in
+        // the median and 23.5 at most (the step: 27.3 us, now 23.5).
         int32_t i = threadIdx.x >> 5, batch = -1;
         const int32_t last_batch = (sh.cta.units - 1) / kBatch;
         auto run_batch = [&](int32_t k) {
@@ -1312,12 +1345,13 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
             if (__shfl_sync(kFull, left, 0) == 1)        // every block was summed before
                 batch = last_batch;
         }
+        bool owes = false;                               // left a batch, and takes one before its next turn
         while (i < turns || (kDense && batch >= 0)) {
             int32_t next = turns, done = -1;
             Block follow = cur;
             if (!kDense || i < turns) {
                 // the next block's index and table entry travel under this one's stream
-                if (batch < 0) {
+                if (kDense ? batch < 0 : !owes) {
                     if (lane == 0)
                         next = atomicAdd(&sh.next, 1);
                     next = __shfl_sync(kFull, next, 0);
@@ -1360,25 +1394,57 @@ gnmr_step_kernel(const __grid_constant__ StepParams p)
                 if (Shape<V>::kGroups ? __any_sync(kFull, left == 1) : __shfl_sync(kFull, left, 0) == 1)
                     done = static_cast<int32_t>(__shfl_sync(kFull, in, 0));
             }
-            if (next >= turns) {
-                __threadfence_block();
-                if (batch < 0) {
+            if constexpr (kDense) {
+                // one batch a CTA or a few: kept by the warp that completes it
+                if (next < turns) {
                     batch = done;
-                    done = -1;
+                    cur = follow;
+                } else {
+                    __threadfence_block();
+                    if (batch < 0) {
+                        batch = done;
+                        done = -1;
+                    }
+                    while (batch >= 0) {
+                        run_batch(batch);
+                        batch = done;
+                        done = -1;
+                    }
+                    if (lane == 0)
+                        next = atomicAdd(&sh.next, 1);
+                    next = __shfl_sync(kFull, next, 0);
+                    if (next < turns)
+                        cur = turn_entry<V>(p, first_turn + next, lane);
                 }
-                while (batch >= 0) {
-                    run_batch(batch);
-                    batch = done;
-                    done = -1;
-                }
-                if (lane == 0)
-                    next = atomicAdd(&sh.next, 1);
-                next = __shfl_sync(kFull, next, 0);
-                if (next < turns)
-                    cur = turn_entry<V>(p, first_turn + next, lane);
             } else {
-                batch = done;
-                cur = follow;
+                if (done >= 0 && (next < turns || owes)) {
+                    leave_batch(sh, done, lane);
+                    done = -1;
+                    owes = true;
+                }
+                if (next < turns) {
+                    cur = follow;
+                } else {
+                    __threadfence_block();
+                    for (;;) {
+                        const int32_t k = done >= 0 ? done : take_batch(sh, lane);
+                        done = -1;
+                        if (k >= 0)
+                            run_batch(k);
+                        if (owes) {
+                            owes = false;
+                            if (lane == 0)
+                                next = atomicAdd(&sh.next, 1);
+                            next = __shfl_sync(kFull, next, 0);
+                            if (next < turns) {
+                                cur = turn_entry<V>(p, first_turn + next, lane);
+                                break;
+                            }
+                        } else if (k < 0) {
+                            break;
+                        }
+                    }
+                }
             }
             i = next;
         }
