@@ -227,17 +227,17 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
     }
     int64_t ctas = std::min<int64_t>(max_ctas, std::max<int64_t>(1, cost / kMinCtaBytes));
     std::vector<int64_t> targets;
-    const bool whole = cost <= max_ctas * kSmallArenaCtaBytes;
-    if (whole)
+    bool cut_at = cost <= max_ctas * kSmallArenaCtaBytes;    // the runs end at `targets`
+    if (cut_at)
         targets = whole_unit_targets(num_segments, seg_lengths, seg_unit, elem_bytes, std::max(kMinCtaBytes, cost / max_ctas));
     const int64_t granule = kSplitBytes / elem_bytes;
     // Few long units per CTA: blocks that make whole turns of its warps.
     const int64_t share = cost / ctas / kWarpsPerCta;
-    const bool even = !whole && cost / num_units >= kEvenUnitBytes && share >= kMinBlockBytes;
+    const bool even = !cut_at && cost / num_units >= kEvenUnitBytes && share >= kMinBlockBytes;
     const int64_t rounds = (share + kEvenBlockBytes - 1) / kEvenBlockBytes;
     for (int64_t bytes = even ? (share + rounds - 1) / rounds : kMinBlockBytes;;) {
         if (ctas > INT32_MAX / 2 || !plan_partition(num_segments, seg_lengths, seg_unit, num_units, elem_bytes,
-                                                    static_cast<int32_t>(ctas), out, whole ? &targets : nullptr))
+                                                    static_cast<int32_t>(ctas), out, cut_at ? &targets : nullptr))
             return false;
         blocks.cta.clear();
         blocks.block.clear();
@@ -293,10 +293,22 @@ bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t
             group_blocks(blocks, elem_bytes);
             return true;
         }
-        if (bytes < kMaxBlockBytes)
+        if (bytes < kMaxBlockBytes) {
             bytes *= 2;
-        else
-            ctas *= 2;
+        } else {
+            // Equal parts, ever smaller: a block costs two bytes and more, so parts of
+            // 4 KB hold few enough however many the segments of a unit.
+            ctas = std::max<int64_t>(2 * ctas, out.num_runs + 1);
+            int64_t points = int64_t(num_units) * kUnitCostBytes;
+            for (int64_t g = 0; g < num_segments; ++g)
+                points += std::max<int64_t>(seg_lengths[g], 1) * elem_bytes;
+            if (ctas > points)
+                return false;                            // unreachable: a run for each byte
+            targets.resize(ctas - 1);
+            for (int64_t w = 1; w < ctas; ++w)
+                targets[w - 1] = static_cast<int64_t>(static_cast<__int128>(points) * w / ctas);
+            cut_at = true;
+        }
     }
 }
 

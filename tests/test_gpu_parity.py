@@ -791,6 +791,31 @@ def test_block_loop_layouts(name, dtype, cuda_device):
             torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("units,segments,most", [(1, 3000, 0), (1, 20_001, 2), (2, 100_000, 1), (300, 400_000, 3)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_block_loop_of_many_tiny_segments(units, segments, most, dtype, cuda_device):
+    """Units of more tiny segments than a CTA has slots for block sums, in
+    arenas small enough to be cut between units: the plan cuts inside them."""
+    import torch
+    rng = np.random.default_rng(segments)
+    lengths = rng.integers(0, most + 1, segments)
+    unit = np.arange(segments) * units // segments
+    offsets = np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64) + 1
+    n = int(lengths.sum()) + 1
+    ids = torch.from_numpy(np.repeat(unit, lengths)).to(cuda_device)
+    with Monitor(offsets, lengths, dtype=dtype, segment_unit=unit.astype(np.int32), num_units=units,
+                 loop_shape="small", window=2) as mon:
+        stats = mon.new_stats()
+        for seed in (1, 2):
+            g = torch.Generator(cuda_device).manual_seed(seed)
+            arena = torch.randn(n, device=cuda_device, generator=g).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+            mon.step(arena, stats=stats)
+            want = torch.zeros(units, dtype=torch.float64, device=cuda_device)
+            want.index_add_(0, ids, arena[1:].double().square())
+            # two roundings of 2^-24 or fewer per segment of up to three elements
+            torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=2.0 ** -23, atol=0)
+
+
 @pytest.mark.parametrize("shape", ["small", "large"])
 @pytest.mark.parametrize("power", [-75, -51, -50, -49, -3, 0, 40, 48, 49, 50, 51, 62])
 def test_lane_totals_of_any_size(power, shape, cuda_device):
