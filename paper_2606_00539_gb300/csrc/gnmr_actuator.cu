@@ -488,6 +488,8 @@ struct HeldRow {
                                           int group, int gl) const
     {
         const bool kept = row_kept(f, mbits);
+        if (kept && src == dst)
+            return;                               // in place: there already
         const float inv = f.fmax / __uint_as_float(mbits);
         const float scale = __uint_as_float(mbits) / f.fmax;
         uint4 *vd = reinterpret_cast<uint4 *>(dst + head * kEB);
@@ -592,6 +594,8 @@ __global__ void __launch_bounds__(kThreads, kLong ? kLongCtas : kShortCtas) fake
             seek(cur, r, t, lane);
             cur.f = (mask != nullptr && mask[cur.unit]) ? rec : low;
         }
+        if (cur.f.code == 0 && in == out)
+            continue;                             // a unit left as it is, in place
         const int64_t n = t.cols[cur.unit];
         const int group = group_of(n, Act<DT>::kN, t.most);
         const int64_t at = (r - cur.begin) * rows_of(group);   // the tile's first row in its unit
