@@ -58,9 +58,11 @@ struct gnmr_actuator {
     int32_t device = 0;
     int32_t sms = 1;
     bool any_long = false;                // some row is too long to be held
+    bool any_held = false;                // and some is not
+    bool by_warp = false;                 // tiles of a warp, not of a CTA
     int32_t most = 0;                     // widest group that holds a row
     int64_t tiles = 0;
-    int64_t tiles_plain = 0;              // tiles of one row per warp
+    int64_t tiles_plain = 0;              // one row each
     int64_t max_end = 0;
     void *dmem = nullptr;
     const int64_t *offset = nullptr;      // [U]
@@ -136,10 +138,10 @@ template <> struct Act<0> {                     // fp32: 4 per vector
     static constexpr int kN = 4;
     __device__ static float load(const void *p, int64_t i) { return static_cast<const float *>(p)[i]; }
     __device__ static void store(void *p, int64_t i, float y) { static_cast<float *>(p)[i] = y; }
-    __device__ static void copy(const void *s, void *d, int64_t i)
-    {
-        static_cast<unsigned int *>(d)[i] = static_cast<const unsigned int *>(s)[i];
-    }
+    using Bits = unsigned int;
+    __device__ static Bits bits(const void *s, int64_t i) { return static_cast<const Bits *>(s)[i]; }
+    __device__ static void put(void *d, int64_t i, Bits x) { static_cast<Bits *>(d)[i] = x; }
+    __device__ static void copy(const void *s, void *d, int64_t i) { put(d, i, bits(s, i)); }
     __device__ static void unpack(const uint4 v, float *x)
     {
         x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y);
@@ -161,10 +163,10 @@ template <> struct Act<1> {                     // bf16: 8 per vector
     {
         static_cast<unsigned short *>(p)[i] = __bfloat16_as_ushort(__float2bfloat16_rn(y));
     }
-    __device__ static void copy(const void *s, void *d, int64_t i)
-    {
-        static_cast<unsigned short *>(d)[i] = static_cast<const unsigned short *>(s)[i];
-    }
+    using Bits = unsigned short;
+    __device__ static Bits bits(const void *s, int64_t i) { return static_cast<const Bits *>(s)[i]; }
+    __device__ static void put(void *d, int64_t i, Bits x) { static_cast<Bits *>(d)[i] = x; }
+    __device__ static void copy(const void *s, void *d, int64_t i) { put(d, i, bits(s, i)); }
     __device__ static void unpack(const uint4 v, float *x)
     {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -221,7 +223,7 @@ template <int DT> __device__ __forceinline__ uint32_t elem_max_bits(const char *
     return __float_as_uint(Act<DT>::load(p, i)) & 0x7fffffffu;
 }
 
-// The rows of a unit are taken in tiles of rows_of(row length); the last tile
+// The rows of a unit are taken in tiles of rows_of(group); the last tile
 // of a unit may hold fewer.  start[b]: first tile of unit b, [U + 1].
 struct RowTables {
     const int64_t *offset;
@@ -341,14 +343,69 @@ __device__ __forceinline__ bool row_kept(const FqFmt &f, uint32_t mbits)
     return f.code == 0 || mbits == 0u || mbits >= 0x7f800000u || isinf(f.fmax / __uint_as_float(mbits));
 }
 
+// Elements [from, to) of a row one by one, kElemLoads in flight per lane (the
+// compiler does not move a load over the stores before it: rows whose input and
+// output lie differently in their 16-byte words are 2-3 times as fast as with
+// one load a lane).
+constexpr int kElemLoads = 16;
+template <int DT> __device__ __forceinline__ uint32_t max_elems(const char *src, int64_t from, int64_t to, int lane)
+{
+    uint32_t m = 0;
+    int64_t i = from + lane;
+    for (; i + (kElemLoads - 1) * 32 < to; i += kElemLoads * 32) {
+        uint32_t x[kElemLoads];
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            x[j] = elem_max_bits<DT>(src, i + j * 32);
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            m = max(m, x[j]);
+    }
+    for (; i < to; i += 32)
+        m = max(m, elem_max_bits<DT>(src, i));
+    return m;
+}
+template <int DT, int CODE>
+__device__ __forceinline__ void quantize_elems(const char *src, char *dst, int64_t from, int64_t to, float inv,
+                                               float scale, int lane)
+{
+    int64_t i = from + lane;
+    for (; i + (kElemLoads - 1) * 32 < to; i += kElemLoads * 32) {
+        float x[kElemLoads];
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            x[j] = Act<DT>::load(src, i + j * 32);
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            Act<DT>::store(dst, i + j * 32, fq_round2<CODE>(x[j] * inv, 0.f).x * scale);
+    }
+    for (; i < to; i += 32)
+        Act<DT>::store(dst, i, fq_round2<CODE>(Act<DT>::load(src, i) * inv, 0.f).x * scale);
+}
+template <int DT>
+__device__ __forceinline__ void copy_elems(const char *src, char *dst, int64_t from, int64_t to, int lane)
+{
+    int64_t i = from + lane;
+    for (; i + (kElemLoads - 1) * 32 < to; i += kElemLoads * 32) {
+        typename Act<DT>::Bits x[kElemLoads];
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            x[j] = Act<DT>::bits(src, i + j * 32);
+#pragma unroll
+        for (int j = 0; j < kElemLoads; ++j)
+            Act<DT>::put(dst, i + j * 32, x[j]);
+    }
+    for (; i < to; i += 32)
+        Act<DT>::copy(src, dst, i);
+}
+
 // Pass 2 of one row in format CODE (one warp): quantize and write.
 template <int DT, int CODE>
 __device__ __forceinline__ void quantize_row_warp(const char *src, char *dst, const uint4 *vs, uint4 *vd,
                                                   int64_t head, int64_t nvec, int64_t tail_at, int64_t n,
                                                   float inv, float scale, int lane)
 {
-    for (int64_t i = lane; i < head; i += 32)
-        Act<DT>::store(dst, i, fq_round2<CODE>(Act<DT>::load(src, i) * inv, 0.f).x * scale);
+    quantize_elems<DT, CODE>(src, dst, 0, head, inv, scale, lane);
     int64_t i = lane;
     for (; i + (kPass2Loads - 1) * 32 < nvec; i += kPass2Loads * 32) {
         uint4 v[kPass2Loads];
@@ -361,8 +418,7 @@ __device__ __forceinline__ void quantize_row_warp(const char *src, char *dst, co
     }
     for (; i < nvec; i += 32)
         st_once(vd + i, quantize_vec<DT, CODE>(ld_last(vs + i), inv, scale));
-    for (int64_t t = tail_at + lane; t < n; t += 32)
-        Act<DT>::store(dst, t, fq_round2<CODE>(Act<DT>::load(src, t) * inv, 0.f).x * scale);
+    quantize_elems<DT, CODE>(src, dst, tail_at, n, inv, scale, lane);
 }
 
 // A row too long for registers, or whose input and output lie differently in
@@ -375,9 +431,7 @@ __device__ __forceinline__ void row_two_pass(const RowRef &q, int lane)
     constexpr int kEB = Act<DT>::kBytes;
     const uint4 *vs = reinterpret_cast<const uint4 *>(q.src + q.head * kEB);
     uint4 *vd = reinterpret_cast<uint4 *>(q.dst + q.head * kEB);
-    uint32_t mbits = 0;
-    for (int64_t i = lane; i < q.head; i += 32)
-        mbits = max(mbits, elem_max_bits<DT>(q.src, i));
+    uint32_t mbits = max_elems<DT>(q.src, 0, q.head, lane);
     int64_t i = lane;
     for (; i + (kPass1Loads - 1) * 32 < q.nvec; i += kPass1Loads * 32) {
         uint4 v[kPass1Loads];
@@ -390,18 +444,15 @@ __device__ __forceinline__ void row_two_pass(const RowRef &q, int lane)
     }
     for (; i < q.nvec; i += 32)
         mbits = max(mbits, vec_max_bits<DT>(ld_keep(vs + i)));
-    for (int64_t t = q.tail_at + lane; t < q.n; t += 32)
-        mbits = max(mbits, elem_max_bits<DT>(q.src, t));
+    mbits = max(mbits, max_elems<DT>(q.src, q.tail_at, q.n, lane));
     mbits = __reduce_max_sync(kFull, mbits);
 
     if (row_kept(q.f, mbits)) {
         if (q.src != q.dst) {
-            for (int64_t t = lane; t < q.head; t += 32)
-                Act<DT>::copy(q.src, q.dst, t);
+            copy_elems<DT>(q.src, q.dst, 0, q.head, lane);
             for (int64_t t = lane; t < q.nvec; t += 32)
                 st_once(vd + t, ld_last(vs + t));
-            for (int64_t t = q.tail_at + lane; t < q.n; t += 32)
-                Act<DT>::copy(q.src, q.dst, t);
+            copy_elems<DT>(q.src, q.dst, q.tail_at, q.n, lane);
         }
         return;
     }
@@ -435,8 +486,14 @@ __host__ __device__ constexpr int group_of(int64_t n, int per_vec, int most)
 constexpr int kWideGroup = 64;
 constexpr int64_t kManyRows = 8;
 static_assert(kThreads == 256, "a row is held by at most eight warps");
-// Rows of one unit that a CTA takes at a time.
-__host__ __device__ constexpr int rows_of(int group) { return group ? kThreads / group : kWarps; }
+// Rows of one unit that a CTA takes at a time.  With kWarpTiles each warp takes
+// rows by itself: where every row is read twice, and in layouts of units of so
+// few rows that more than half of the warps of CTA tiles would have none, if no
+// row takes more than a warp (1,000 units of one 64-element row 7.9 -> 3.9 us).
+template <bool kWarpTiles> __host__ __device__ constexpr int rows_of(int group)
+{
+    return group ? (kWarpTiles ? 32 : kThreads) / group : kWarpTiles ? 1 : kWarps;
+}
 
 // A row of n elements (0: none) held by a group of threads, `gl` the thread's
 // place in it: vector gl + group j in v[j], and of the head and the tail (less
@@ -529,13 +586,13 @@ struct GroupMax {
     uint32_t slot[3][2][kWarps];
 };
 
-// One tile of held rows: the CTA's threads in groups, one row each.  `turn`
+// One tile of held rows: the CTA's (or warp's) threads in groups, one row each.  `turn`
 // has a bit for each width, the set of slots it uses next.
-template <int DT>
+template <int DT, bool kWarpTiles>
 __device__ __forceinline__ void held_tile(const char *src, char *dst, int n, int group, int count, const FqFmt &f,
                                           GroupMax &gm, uint32_t &turn)
 {
-    const int row = threadIdx.x >> (__ffs(group) - 1), gl = threadIdx.x & (group - 1);
+    const int row = (kWarpTiles ? threadIdx.x & 31 : threadIdx.x) >> (__ffs(group) - 1), gl = threadIdx.x & (group - 1);
     const bool there = row < count;
     const int64_t at = there ? static_cast<int64_t>(row) * n * Act<DT>::kBytes : 0;
     src += at;
@@ -545,7 +602,7 @@ __device__ __forceinline__ void held_tile(const char *src, char *dst, int n, int
     uint32_t m = h.max_bits();
     if (group >= 32) {
         m = __reduce_max_sync(kFull, m);
-        if (group > 32) {
+        if (!kWarpTiles && group > 32) {
             const int warps = group / 32, first = row * warps;
             const int width = warps == 2 ? 0 : warps == 4 ? 1 : 2;
             const int barrier = (width == 0 ? 1 : width == 1 ? 5 : 7) + row;     // 1-4, 5-6, 7
@@ -570,9 +627,9 @@ __device__ __forceinline__ void held_tile(const char *src, char *dst, int n, int
     }
 }
 
-// kLong = false: every row is held.  Held rows need input and output to share
+// kLong = false: every row is held; kLong and kWarpTiles: none.  Held rows need input and output to share
 // their 16-byte alignment (the host sees to it: most = 0 where they do not).
-template <int DT, bool kLong>
+template <int DT, bool kLong, bool kWarpTiles>
 __global__ void __launch_bounds__(kThreads, kLong ? kLongCtas : kShortCtas) fake_quant_kernel(
     const void *in, void *out, RowTables t, const uint8_t *mask, FqFmt low, FqFmt rec)
 {
@@ -580,7 +637,11 @@ __global__ void __launch_bounds__(kThreads, kLong ? kLongCtas : kShortCtas) fake
     __shared__ GroupMax s_max;
     uint32_t turn = 0;
     const int lane = threadIdx.x & 31;
-    int64_t r = blockIdx.x;
+    int64_t r = blockIdx.x, stride = gridDim.x;
+    if (kWarpTiles) {
+        r += stride * (threadIdx.x >> 5);
+        stride *= kWarps;
+    }
     UnitCursor cur;
     // The tables never change after create: the first unit is looked up while
     // the kernel before this one on the stream is still running.  Its writes
@@ -589,7 +650,7 @@ __global__ void __launch_bounds__(kThreads, kLong ? kLongCtas : kShortCtas) fake
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     cur.f = (mask != nullptr && mask[cur.unit]) ? rec : low;
-    for (; r < t.tiles; r += gridDim.x) {
+    for (; r < t.tiles; r += stride) {
         if (r >= cur.end) {
             seek(cur, r, t, lane);
             cur.f = (mask != nullptr && mask[cur.unit]) ? rec : low;
@@ -597,25 +658,29 @@ __global__ void __launch_bounds__(kThreads, kLong ? kLongCtas : kShortCtas) fake
         if (cur.f.code == 0 && in == out)
             continue;                             // a unit left as it is, in place
         const int64_t n = t.cols[cur.unit];
-        const int group = group_of(n, Act<DT>::kN, t.most);
-        const int64_t at = (r - cur.begin) * rows_of(group);   // the tile's first row in its unit
+        const int group = kLong && kWarpTiles ? 0 : group_of(n, Act<DT>::kN, t.most);
+        const int rows = rows_of<kWarpTiles>(group);
+        const int64_t at = (r - cur.begin) * rows;             // the tile's first row in its unit
         const int64_t e0 = t.offset[cur.unit] + at * n;
         const int64_t left = t.rows[cur.unit] - at;
-        const int count = left < rows_of(group) ? static_cast<int>(left) : rows_of(group);
+        const int count = left < rows ? static_cast<int>(left) : rows;
         if (kLong) {
             if (group == 0) {
-                for (int k = threadIdx.x >> 5; k < count; k += kWarps)
+                const int k = kWarpTiles ? 0 : threadIdx.x >> 5;
+                if (k < count)
                     row_two_pass<DT>(locate_row<DT>(e0 + k * n, n, cur.f, in, out), lane);
                 continue;
             }
         }
-        held_tile<DT>(static_cast<const char *>(in) + e0 * kEB, static_cast<char *>(out) + e0 * kEB,
+        if (kLong && kWarpTiles)
+            continue;
+        held_tile<DT, kWarpTiles>(static_cast<const char *>(in) + e0 * kEB, static_cast<char *>(out) + e0 * kEB,
                       static_cast<int>(n), group, count, cur.f, s_max, turn);
     }
 }
 
 // Launched as a programmatic dependent of the kernel before it on the stream.
-template <int DT, bool kLong>
+template <int DT, bool kLong, bool kWarpTiles>
 cudaError_t launch_shape(const RowTables &t, int sms, const void *in, void *out, const uint8_t *mask, FqFmt low,
                          FqFmt rec, cudaStream_t stream)
 {
@@ -628,7 +693,7 @@ cudaError_t launch_shape(const RowTables &t, int sms, const void *in, void *out,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fake_quant_kernel<DT, kLong>, in, out, t, mask, low, rec);
+    return cudaLaunchKernelEx(&cfg, fake_quant_kernel<DT, kLong, kWarpTiles>, in, out, t, mask, low, rec);
 }
 
 template <int DT>
@@ -637,14 +702,17 @@ cudaError_t launch(const gnmr_actuator &a, const void *in, void *out, const uint
 {
     const bool together = ((reinterpret_cast<uintptr_t>(in) ^ reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
     RowTables t{a.offset, a.rows, a.cols, a.start, a.tiles, a.num_units, a.most};
-    if (together && !a.any_long)
-        return launch_shape<DT, false>(t, a.sms, in, out, mask, low, rec, stream);
-    if (!together) {                              // no common vectors: every row element by element
-        t.start = a.start_plain;
-        t.tiles = a.tiles_plain;
-        t.most = 0;
+    if (together && a.any_held) {
+        if (a.any_long)
+            return launch_shape<DT, true, false>(t, a.sms, in, out, mask, low, rec, stream);
+        return a.by_warp ? launch_shape<DT, false, true>(t, a.sms, in, out, mask, low, rec, stream)
+                         : launch_shape<DT, false, false>(t, a.sms, in, out, mask, low, rec, stream);
     }
-    return launch_shape<DT, true>(t, a.sms, in, out, mask, low, rec, stream);
+    // every row read twice: too long, or no 16-byte vectors in common
+    t.start = a.start_plain;
+    t.tiles = a.tiles_plain;
+    t.most = 0;
+    return launch_shape<DT, true, true>(t, a.sms, in, out, mask, low, rec, stream);
 }
 
 gnmr_status act_fail(gnmr_status s, const std::string &why)
@@ -695,7 +763,20 @@ gnmr_status gnmr_actuator_create(int32_t num_units, const int64_t *offsets, cons
         if (group_of(cols[b], per_vec, kWideGroup) == 0)
             wide += rows[b];
     const int most = wide < kManyRows * sms * kLongCtas * kWarps ? kThreads : kWideGroup;
-    bool any_long = false;
+    bool any_long = false, any_held = false, by_warp = true;
+    int64_t cta_tiles = 0, warp_tiles = 0;
+    const auto tiles_of = [](int64_t n, int64_t per) { return n / per + (n % per != 0); };
+    for (size_t b = 0; b < U; ++b) {
+        const int group = group_of(cols[b], per_vec, most);
+        any_long |= group == 0 && rows[b] > 0;
+        any_held |= group != 0 && rows[b] > 0;
+        by_warp &= group != 0 && group <= 32;
+        if (by_warp) {
+            cta_tiles += tiles_of(rows[b], rows_of<false>(group));
+            warp_tiles += tiles_of(rows[b], rows_of<true>(group));
+        }
+    }
+    by_warp &= cta_tiles * kWarps > 2 * warp_tiles;
     std::vector<int64_t> img;
     try {
         img.resize(5 * U + 2);
@@ -711,10 +792,8 @@ gnmr_status gnmr_actuator_create(int32_t num_units, const int64_t *offsets, cons
     start[0] = start_plain[0] = 0;
     for (size_t b = 0; b < U; ++b) {
         const int group = group_of(cols[b], per_vec, most);
-        any_long |= group == 0 && rows[b] > 0;
-        const int64_t per = rows_of(group);
-        start[b + 1] = start[b] + rows[b] / per + (rows[b] % per != 0);
-        start_plain[b + 1] = start_plain[b] + rows[b] / kWarps + (rows[b] % kWarps != 0);
+        start[b + 1] = start[b] + tiles_of(rows[b], by_warp ? rows_of<true>(group) : rows_of<false>(group));
+        start_plain[b + 1] = start_plain[b] + rows[b];
     }
     cudaError_t e = cudaMalloc(&a->dmem, 8 * img.size());
     if (e == cudaSuccess)
@@ -743,6 +822,8 @@ gnmr_status gnmr_actuator_create(int32_t num_units, const int64_t *offsets, cons
     a->tiles_plain = start_plain[U];
     a->max_end = max_end;
     a->any_long = any_long;
+    a->any_held = any_held;
+    a->by_warp = by_warp;
     a->sms = sms;
     *out = a;
     return GNMR_OK;

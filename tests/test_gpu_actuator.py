@@ -259,3 +259,38 @@ def test_units_kept_in_place(dtype, cuda_device):
         assert np.array_equal(_host_bits(x).view(word), host.view(word))
     finally:
         N.gnmr_actuator_destroy(h)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("most_rows", [1, 3])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_units_of_few_rows(dtype, most_rows, shift, cuda_device):
+    """Units of a few short rows, which warps take one by one: rows of up to a
+    warp's 256 vectors, empty units among them, against the oracle."""
+    import torch
+    rng = np.random.default_rng(most_rows)
+    per = 8 if dtype == "bf16" else 4
+    cols = np.array([1, per, 33 * per, 64 * per - 1, 129 * per, 256 * per + per - 1, 31] * 40, np.int64)
+    rows = rng.integers(0, most_rows + 1, len(cols)).astype(np.int64)
+    rows[0] = 1
+    off = np.concatenate([[0], np.cumsum(rows * cols + 1)[:-1]]).astype(np.int64)
+    total = int(off[-1] + rows[-1] * cols[-1]) + 1
+    g = torch.Generator(cuda_device).manual_seed(most_rows)
+    x = torch.randn(total, device=cuda_device, generator=g).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    x[off[14]:off[14] + rows[14] * cols[14]] = 0
+    out = torch.zeros(total + 16, dtype=x.dtype, device=cuda_device)[shift:shift + total]
+    mask = (np.arange(len(rows)) % 3 == 0).astype(np.uint8)
+    d_mask = torch.from_numpy(mask).to(cuda_device)
+    h = N.gnmr_actuator_create(off, rows, cols, N.GNMR_DTYPE_BF16 if dtype == "bf16" else N.GNMR_DTYPE_F32, 0)
+    try:
+        low, rec = N.GNMR_FQ_E2M1, N.GNMR_FQ_E4M3
+        N.gnmr_actuator_apply(h, x.data_ptr(), out.data_ptr(), total, d_mask.data_ptr(), low, rec)
+        torch.cuda.synchronize()
+        want = _oracle_apply(_host_bits(x), off, rows, cols, [rec if m else low for m in mask])
+        got = _host_bits(out)
+        word = np.uint16 if dtype == "bf16" else np.uint32
+        for b in range(len(rows)):
+            part = slice(off[b], off[b] + rows[b] * cols[b])
+            assert np.array_equal(got[part].view(word), want[part].view(word)), (b, rows[b], cols[b])
+    finally:
+        N.gnmr_actuator_destroy(h)
