@@ -38,8 +38,10 @@ constexpr int64_t kMaxUnits = int64_t(1) << 17;        // 131,072 units
 constexpr int64_t kMaxWarps = int64_t(1) << 14;        // streaming warps of one call
 // Gradient bytes per chunk, the granularity at which warp ranges are cut: fine,
 // or so coarse that a layout of small units is not cut inside a unit at all
-// (then no ticket has to be cleared, which saves a launch).
+// (then no ticket has to be taken or cleared, which saves a launch: 2,048 fp32
+// units of 6 to 18 KB 10.7 -> 6.7 us, 1,000 of 8 to 24 KB 10.4 -> 7.2).
 constexpr int kFineShift = 12, kCoarseShift = 14;      // log2: 4 KiB, 16 KiB
+constexpr int kWholeShift = 15;                        // 32 KiB, where every unit can have its warp
 constexpr int64_t kSpanBytes = int64_t(64) << 10;      // bytes of a unit summed in one go
 constexpr int kThreads = 512;
 constexpr int kWarpsPerCta = kThreads / 32;
@@ -390,9 +392,6 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
             longest = l > longest ? l : longest;
         }
     }
-    const int bytes_shift = longest > (int64_t(1) << kCoarseShift) / eb ? kFineShift : kCoarseShift;
-    const int64_t chunk_bytes = int64_t(1) << bytes_shift;
-    const int chunk_shift = bytes_shift - (eb == 2 ? 1 : 2);   // in elements
     if ((!d_arena && max_end > 0) || reinterpret_cast<uintptr_t>(d_arena) % eb != 0)
         return reject(GNMR_ERR_INVALID_ARG, kErrArena);
 
@@ -405,6 +404,11 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
         return reject(GNMR_ERR_CUDA, kErrCuda);
     if (sms < 1)
         return reject(GNMR_ERR_CUDA, kErrDevice);
+    const int64_t warps = int64_t(sms) * 2 * kWarpsPerCta;     // two resident CTAs per SM
+    const int coarse = num_units <= warps ? kWholeShift : kCoarseShift;
+    const int bytes_shift = longest > (int64_t(1) << coarse) / eb ? kFineShift : coarse;
+    const int64_t chunk_bytes = int64_t(1) << bytes_shift;
+    const int chunk_shift = bytes_shift - (eb == 2 ? 1 : 2);   // in elements
     unsigned char *base = static_cast<unsigned char *>(addr);
     const View v = carve(base);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -418,8 +422,7 @@ extern "C" gnmr_status gnmr_unit_norms_static(const void *d_arena, int64_t arena
             total += gnmr::kUnitCostBytes + lengths[b] * eb;
         }
         g_host_chunk_start[num_units] = T;
-        int64_t want = int64_t(sms) * 2 * kWarpsPerCta;    // two resident CTAs per SM
-        want = want < kMaxWarps ? want : kMaxWarps;
+        int64_t want = warps < kMaxWarps ? warps : kMaxWarps;
         want = want < T ? want : T;
         // cut points: the first chunk starting at or after cost total * k / want
         int64_t nb = 0, k = 1, ucost = 0;

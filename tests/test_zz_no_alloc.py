@@ -160,10 +160,10 @@ def test_static_norms_reject_tables_of_another_layout(cuda_device):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("name", ["uncut", "cut", "spans", "many"])
+@pytest.mark.parametrize("name", ["uncut", "cut", "spans", "many", "whole", "past-whole", "many-cut"])
 def test_static_norms_of_cut_and_uncut_units(dtype, name, cuda_device):
-    """Units up to 16 KiB are never cut (no tickets), longer ones at 4 KiB and
-    summed 64 KiB at a time; a warp finishes more units than its 32 lanes
+    """Units up to 16 KiB, or 32 KiB where every unit can have a warp, are
+    never cut (no tickets), longer ones at 4 KiB and summed 64 KiB at a time; a warp finishes more units than its 32 lanes
     hold.  The same layout again on a shorter arena is rejected, and in the
     other dtype planned anew."""
     import torch
@@ -172,6 +172,9 @@ def test_static_norms_of_cut_and_uncut_units(dtype, name, cuda_device):
     rng = np.random.default_rng(3)
     ln = {"uncut": rng.integers(0, top + 1, 3000), "cut": np.append(rng.integers(0, top, 500), [top + 1, top, top - 1]),
           "spans": np.array([0, 4 * top, 4 * top + 1, 40_000_003, 1, 8 * top - 1, 3]),
+          "whole": np.append(rng.integers(0, 2 * top, 1500), [2 * top, 2 * top - 1, 0]),
+          "past-whole": np.append([2 * top + 1], rng.integers(0, 2 * top, 1500)),
+          "many-cut": np.append(rng.integers(0, top // 4, 6000), [top + 1, 2 * top]),
           "many": rng.integers(0, 3, 131072)}[name].astype(np.int64)
     off = np.concatenate([[0], np.cumsum(ln)[:-1]]).astype(np.int64) + 1
     n = int(ln.sum()) + 1
