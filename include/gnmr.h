@@ -152,16 +152,18 @@ typedef struct gnmr_info {
     int32_t device;
     int32_t num_ctas;          /* CTAs per gnmr_step launch */
     int32_t threads_per_cta;
-    int32_t num_warps;         /* warps with a work run */
-    int64_t num_partials;      /* per-(run, unit) partial sums */
+    int32_t num_warps;         /* warps with work at the start of a launch: a run, or with
+                                  the small-unit loop a block of their CTA's part */
+    int64_t num_partials;      /* partial sums per (run, unit), or (CTA, unit) with the
+                                  small-unit loop */
     int64_t device_bytes;      /* library-owned device memory */
     int64_t arena_elems_min;   /* max over units of offset + length */
     int64_t steps;             /* gnmr_step calls enqueued so far */
     int32_t loop_shape;        /* gnmr_loop_shape in use (never GNMR_LOOP_AUTO) */
-    int32_t num_runs;          /* work runs: one per warp with the small-unit loop;
-                                  about 16 per warp with the large-unit loop, where
-                                  each warp starts on its own and then takes the
-                                  next untaken one */
+    int32_t num_runs;          /* work runs: num_warps with the small-unit loop (whose
+                                  warps take blocks); about 16 per warp with the
+                                  large-unit loop, where each warp starts on its own
+                                  and then takes the next untaken one */
 } gnmr_info;
 
 typedef struct gnmr_handle gnmr_handle;
