@@ -52,9 +52,9 @@ constexpr int64_t kBulkRunMin = int64_t(64) << 10;
 constexpr int64_t kBulkRunMax = int64_t(256) << 10;
 
 // Small-unit loop: every CTA owns a contiguous part of the segment stream of
-// at least kMinCtaBytes of cost, cut into blocks of at most kMinBlockBytes
-// (doubled until a CTA has at most kBlocksPerCta), which its warps take in
-// turn.  kBatch units are one batch of the unit epilogue.  8 KiB blocks, two
+// at least kMinCtaBytes of cost, cut into blocks of at most kMinBlockBytes (or
+// that doubled, up to kMaxBlockBytes, if a CTA would have more than kBlocksPerCta
+// for its bytes alone), which its warps take in turn.  kBatch units are one batch of the unit epilogue.  8 KiB blocks, two
 // load rounds of a warp: 4 KiB took 246.8 us on 100K units, 8 KiB 242.9, 16
 // KiB 244.2 (560 units of 224 KB: 34.1, 32.7, 31.6).  24 KiB per CTA: 3.7 MB
 // over 64 units took 11.9 us with 64 KiB, 11.4 with 24.
@@ -285,8 +285,8 @@ struct BlockPlan {
     bool grouped = false;
 };
 
-// Cuts the stream into one run per CTA (about max_ctas of them, more where a
-// run would hold more than kBlocksPerCta blocks) and the runs into blocks.
+// Cuts the stream into one run per CTA (about max_ctas of them, more where their
+// kBlocksPerCta blocks each do not do) and the runs into blocks.
 // Same input rules as plan_partition; seg_offsets in elements.
 bool plan_blocks(int64_t num_segments, const int64_t *seg_offsets, const int64_t *seg_lengths,
                  const int32_t *seg_unit, int32_t num_units, int elem_bytes, int32_t max_ctas, Plan &out,

@@ -816,6 +816,29 @@ def test_block_loop_of_many_tiny_segments(units, segments, most, dtype, cuda_dev
             torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=2.0 ** -23, atol=0)
 
 
+@pytest.mark.parametrize("tiny,large,where", [(2500, 400, 0), (5000, 400, 200), (100_000, 300, 300)])
+def test_block_loop_of_tiny_segments_among_large_units(tiny, large, where, cuda_device):
+    """A unit of more one-element segments than a CTA has slots for block sums,
+    before, between or after ordinary units: it alone is cut shorter."""
+    import torch
+    lengths = np.concatenate([np.full(where, 100_001), np.ones(tiny, np.int64), np.full(large - where, 100_001)])
+    unit = np.concatenate([np.arange(where), np.full(tiny, where), np.arange(where + 1, large + 1)])
+    offsets = np.cumsum(lengths) - lengths
+    ids = torch.from_numpy(np.repeat(unit, lengths)).to(cuda_device)
+    with Monitor(offsets, lengths, dtype="f32", segment_unit=unit.astype(np.int32), num_units=large + 1,
+                 loop_shape="small", window=2) as mon:
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert mon.info()["num_ctas"] <= (2 if tiny <= 5000 else 4) * sms
+        stats = mon.new_stats()
+        g = torch.Generator(cuda_device).manual_seed(tiny)
+        arena = torch.randn(int(lengths.sum()), device=cuda_device, generator=g)
+        mon.step(arena, stats=stats)
+        want = torch.zeros(large + 1, dtype=torch.float64, device=cuda_device).index_add_(0, ids, arena.double().square())
+        # at most 27 fp32 roundings per block of 16 iterations, and 2^-26 per lane
+        torch.testing.assert_close(stats["norm"], want.sqrt(), rtol=1e-6, atol=0)
+        assert torch.equal(mon.step_partials(arena).sqrt(), stats["norm"])
+
+
 @pytest.mark.parametrize("shape", ["small", "large"])
 @pytest.mark.parametrize("power", [-75, -51, -50, -49, -3, 0, 40, 48, 49, 50, 51, 62])
 def test_lane_totals_of_any_size(power, shape, cuda_device):
