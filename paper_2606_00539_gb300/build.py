@@ -20,7 +20,7 @@ LIB_PATH = os.path.join(PKG, "libgnmr.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CUDA_SOURCES = ["gnmr_kernels.cu", "gnmr_static.cu", "gnmr_actuator.cu"]
 CXX_SOURCES = ["gnmr_api.cpp", "gnmr_plan.cpp"]
-HEADERS = ["gnmr_internal.h"]
+HEADERS = ["gnmr_internal.h", "gnmr_stream.cuh"]
 
 
 def _cuda_home() -> str:

@@ -161,6 +161,15 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
         N.load()
 
 
+def test_every_source_makes_the_library_stale():
+    """Each file that the library is compiled from, included ones too, counts
+    when is_stale() asks whether it has to be built again."""
+    inputs = {os.path.realpath(f) for f in native_build._inputs()}
+    for folder in (native_build.CSRC, native_build.INCLUDE):
+        for name in os.listdir(folder):
+            assert os.path.realpath(os.path.join(folder, name)) in inputs, name
+
+
 # ---------------------------------------------------------------------------
 # Work partition (host logic of gnmr_create)
 # ---------------------------------------------------------------------------
