@@ -323,17 +323,19 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
             delete h;
             return fail_create(GNMR_ERR_INVALID_ARG, "work partition failed (sizes out of range)");
         }
-        const int64_t W = plan.num_runs;
+        // the large-unit loop reads segments and runs, the small-unit loop blocks
+        const bool by_run = variant == gnmr::kVariantBulk;
+        const size_t SR = by_run ? S : 0, UR = by_run ? U : 0, WR = by_run ? plan.num_runs + 1 : 0;
         Carver cv;
-        const size_t o_off = cv.take(sizeof(int64_t) * S);
-        const size_t o_len = cv.take(sizeof(int64_t) * S);
-        const size_t o_segu = cv.take(sizeof(int32_t) * S);
+        const size_t o_off = cv.take(sizeof(int64_t) * SR);
+        const size_t o_len = cv.take(sizeof(int64_t) * SR);
+        const size_t o_segu = cv.take(sizeof(int32_t) * SR);
         const size_t o_rec = cv.take(U);
-        const size_t o_run_seg = cv.take(sizeof(int64_t) * (W + 1));
-        const size_t o_run_pos = cv.take(sizeof(int64_t) * (W + 1));
-        const size_t o_first = cv.take(sizeof(int32_t) * U);
-        const size_t o_parts = cv.take(sizeof(int32_t) * U);
-        const size_t o_pbase = cv.take(sizeof(int64_t) * U);
+        const size_t o_run_seg = cv.take(sizeof(int64_t) * WR);
+        const size_t o_run_pos = cv.take(sizeof(int64_t) * WR);
+        const size_t o_first = cv.take(sizeof(int32_t) * UR);
+        const size_t o_parts = cv.take(sizeof(int32_t) * UR);
+        const size_t o_pbase = cv.take(sizeof(int64_t) * UR);
         const size_t o_partial = cv.take(sizeof(double) * plan.num_partials);
         const size_t o_ticket = cv.take(sizeof(uint32_t) * U);
         const size_t o_state = cv.take(sizeof(gnmr::UnitState) * U);
@@ -350,9 +352,20 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
 
         // Host image of the whole block: static tables plus zeroed state.
         std::vector<unsigned char> img(cv.size, 0);
-        std::memcpy(&img[o_off], seg_off.data(), sizeof(int64_t) * S);
-        std::memcpy(&img[o_len], seg_len.data(), sizeof(int64_t) * S);
-        std::memcpy(&img[o_segu], seg_unit.data(), sizeof(int32_t) * S);
+        if (by_run) {
+            std::memcpy(&img[o_off], seg_off.data(), sizeof(int64_t) * S);
+            std::memcpy(&img[o_len], seg_len.data(), sizeof(int64_t) * S);
+            std::memcpy(&img[o_segu], seg_unit.data(), sizeof(int32_t) * S);
+            std::memcpy(&img[o_run_seg], plan.run_seg.data(), sizeof(int64_t) * WR);
+            std::memcpy(&img[o_run_pos], plan.run_pos.data(), sizeof(int64_t) * WR);
+            std::memcpy(&img[o_first], plan.first_run.data(), sizeof(int32_t) * U);
+            std::memcpy(&img[o_parts], plan.num_parts.data(), sizeof(int32_t) * U);
+            std::memcpy(&img[o_pbase], plan.part_base.data(), sizeof(int64_t) * U);
+        } else {
+            std::memcpy(&img[o_ctab], blocks.cta.data(), sizeof(gnmr::CtaBlocks) * blocks.cta.size());
+            std::memcpy(&img[o_block], blocks.block.data(), sizeof(gnmr::Block) * blocks.block.size());
+            std::memcpy(&img[o_ublock], blocks.unit_block.data(), sizeof(int32_t) * blocks.unit_block.size());
+        }
         int32_t num_rec = 0;
         for (int64_t b = 0; b < U; ++b) {
             img[o_rec + b] = c.recoverable ? (c.recoverable[b] != 0) : 1;
@@ -360,16 +373,6 @@ gnmr_status gnmr_create(const gnmr_config *cfg, gnmr_handle **out)
         }
         if (c.unit_cost)
             std::memcpy(&img[o_cost], c.unit_cost, sizeof(double) * U);
-        std::memcpy(&img[o_run_seg], plan.run_seg.data(), sizeof(int64_t) * (W + 1));
-        std::memcpy(&img[o_run_pos], plan.run_pos.data(), sizeof(int64_t) * (W + 1));
-        std::memcpy(&img[o_first], plan.first_run.data(), sizeof(int32_t) * U);
-        std::memcpy(&img[o_parts], plan.num_parts.data(), sizeof(int32_t) * U);
-        std::memcpy(&img[o_pbase], plan.part_base.data(), sizeof(int64_t) * U);
-        if (!blocks.cta.empty()) {
-            std::memcpy(&img[o_ctab], blocks.cta.data(), sizeof(gnmr::CtaBlocks) * blocks.cta.size());
-            std::memcpy(&img[o_block], blocks.block.data(), sizeof(gnmr::Block) * blocks.block.size());
-            std::memcpy(&img[o_ublock], blocks.unit_block.data(), sizeof(int32_t) * blocks.unit_block.size());
-        }
         std::memset(&img[o_partial], 0xff, sizeof(double) * plan.num_partials);   // every slot empty
         static_assert(gnmr::kEmptyPartial == ~0ull, "empty partial slots are all-ones bytes");
         {

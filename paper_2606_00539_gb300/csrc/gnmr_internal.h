@@ -193,6 +193,7 @@ inline Divisor make_divisor(double v)
 
 struct StepParams {
     const void *arena;
+    // large-unit loop only (first_run, num_parts and part_base too)
     const int64_t *offset;       // [S] segment offsets, segments grouped by unit
     const int64_t *length;       // [S] segment lengths
     const int32_t *seg_unit;     // [S] unit of each segment (non-decreasing)
@@ -202,7 +203,7 @@ struct StepParams {
     const CtaBlocks *cta_blocks; // [num_ctas] small-unit loop: each CTA's part,
     const Block *block;          // the blocks of all CTAs, in the order the warps take them
     const int32_t *unit_block;   // [U + 1] and the first block of each unit
-    const int32_t *first_run;    // [U] first run (small-unit loop: CTA) touching unit b
+    const int32_t *first_run;    // [U] first run touching unit b
     const int32_t *num_parts;    // [U]
     const int64_t *part_base;    // [U] first partial slot of unit b
     double *partial;             // [num_partials]

@@ -755,6 +755,20 @@ def test_loop_shape_of_small_arenas(mib, extra, want, cuda_device):
         assert mon.info()["loop_shape"] == (N.GNMR_LOOP_LARGE_UNITS if want == "large" else N.GNMR_LOOP_SMALL_UNITS)
 
 
+def test_device_memory_of_a_small_unit_handle(cuda_device):
+    """Per unit: state, window, candidate, ticket, flag, one partial sum, one
+    block and its place; nothing of the large-unit loop's tables."""
+    U, window = 50_000, 2
+    lengths = np.full(U, 1000, np.int64)                  # 4 KB, one block of a whole warp
+    with Monitor(np.cumsum(lengths) - lengths, lengths, dtype="f32", window=window) as mon:
+        info = mon.info()
+    assert info["loop_shape"] == N.GNMR_LOOP_SMALL_UNITS
+    unit = 40 + 8 * window + 16 + 4 + 1 + 8 + 16 + 4
+    cta = 64 + 2 * 8 + 2 * 16                             # table, and the parts of the units it cuts
+    fixed = 16 * 8192 + 4 * 2048 + 256 + 12 * 256         # hot list, histogram, control, alignment
+    assert info["device_bytes"] <= unit * U + cta * info["num_ctas"] + fixed
+
+
 def _block_layout(name):
     if name == "block-edges":                             # around one and two blocks of 8 KiB
         return np.repeat([0, 1, 2047, 2048, 2049, 4095, 4096, 4097, 6145], 40)
