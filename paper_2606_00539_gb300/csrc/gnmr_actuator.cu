@@ -766,14 +766,16 @@ gnmr_status gnmr_actuator_create(int32_t num_units, const int64_t *offsets, cons
     bool any_long = false, any_held = false, by_warp = true;
     int64_t cta_tiles = 0, warp_tiles = 0;
     const auto tiles_of = [](int64_t n, int64_t per) { return n / per + (n % per != 0); };
+    // rows without elements are no work, however many a unit claims to have
+    const auto rows_with = [&](size_t b) { return cols[b] > 0 ? rows[b] : 0; };
     for (size_t b = 0; b < U; ++b) {
         const int group = group_of(cols[b], per_vec, most);
-        any_long |= group == 0 && rows[b] > 0;
-        any_held |= group != 0 && rows[b] > 0;
+        any_long |= group == 0 && rows_with(b) > 0;
+        any_held |= group != 0 && rows_with(b) > 0;
         by_warp &= group != 0 && group <= 32;
         if (by_warp) {
-            cta_tiles += tiles_of(rows[b], rows_of<false>(group));
-            warp_tiles += tiles_of(rows[b], rows_of<true>(group));
+            cta_tiles += tiles_of(rows_with(b), rows_of<false>(group));
+            warp_tiles += tiles_of(rows_with(b), rows_of<true>(group));
         }
     }
     by_warp &= cta_tiles * kWarps > 2 * warp_tiles;
@@ -792,8 +794,8 @@ gnmr_status gnmr_actuator_create(int32_t num_units, const int64_t *offsets, cons
     start[0] = start_plain[0] = 0;
     for (size_t b = 0; b < U; ++b) {
         const int group = group_of(cols[b], per_vec, most);
-        start[b + 1] = start[b] + tiles_of(rows[b], by_warp ? rows_of<true>(group) : rows_of<false>(group));
-        start_plain[b + 1] = start_plain[b] + rows[b];
+        start[b + 1] = start[b] + tiles_of(rows_with(b), by_warp ? rows_of<true>(group) : rows_of<false>(group));
+        start_plain[b + 1] = start_plain[b] + rows_with(b);
     }
     cudaError_t e = cudaMalloc(&a->dmem, 8 * img.size());
     if (e == cudaSuccess)

@@ -211,6 +211,27 @@ def test_actuator_driven_by_gnmr_step(cuda_device):
         mon.close()
 
 
+@pytest.mark.parametrize("where", [0, 1])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_rows_without_elements_take_no_time(where, shift, cuda_device):
+    """A unit of 2^58 rows of no columns has nothing to quantize: its rows are
+    not walked, and the unit beside it comes out as if it were alone."""
+    import torch
+    rows, cols = np.array([5, 5], np.int64), np.array([70, 70], np.int64)
+    rows[where], cols[where] = 1 << 58, 0
+    x = torch.randn(350, device=cuda_device)
+    out = torch.zeros(366, device=cuda_device)[shift:shift + 350]
+    for counts in (rows, np.where(cols > 0, 0, rows)):    # then nothing at all
+        h = N.gnmr_actuator_create(np.zeros(2, np.int64), counts, cols, N.GNMR_DTYPE_F32, 0)
+        try:
+            N.gnmr_actuator_apply(h, x.data_ptr(), out.data_ptr(), 350, None, N.GNMR_FQ_E2M1, N.GNMR_FQ_E4M3)
+            torch.cuda.synchronize()
+        finally:
+            N.gnmr_actuator_destroy(h)
+    want = _oracle_apply(_host_bits(x), np.zeros(1, np.int64), np.array([5]), np.array([70]), [N.GNMR_FQ_E2M1])
+    assert np.array_equal(_host_bits(out), want)
+
+
 def test_actuator_errors(cuda_device):
     import torch
     off = np.array([0, 10], np.int64)
