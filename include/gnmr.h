@@ -284,19 +284,21 @@ const char *gnmr_status_string(gnmr_status s);
  * create on this thread); never NULL. */
 const char *gnmr_last_error(const gnmr_handle *h);
 
-/* Host-only query of the work partition that gnmr_create plans (max_warps =
- * the number of runs asked for; "warp" below stands for whoever streams a
- * run): the concatenation
- * of all units (an empty unit counts as one element of work) is cut into at
- * most max_warps contiguous runs of about equal cost (element bytes plus a
- * fixed per-unit cost).  (The small-unit loop shape cuts into one run per
- * resident CTA, whose warps then share it block by block; the large-unit
- * shape into about 16 runs per warp, see gnmr_info.num_runs.)  Outputs,
- * caller-allocated: run_unit / run_pos [max_warps + 1] (run w covers
- * (run_unit[w], run_pos[w]) up to, not including, (run_unit[w+1],
- * run_pos[w+1])), first_warp / num_parts [num_units] (the warps touching
- * unit b are first_warp[b] .. first_warp[b] + num_parts[b] - 1).  *num_warps
- * receives the number of runs.  No CUDA call is made.  Errors:
+/* Host-only query of the equal-cost cut that gnmr_create's plans start from:
+ * the concatenation of all units (an empty unit counts as one element of work)
+ * is cut into at most max_warps contiguous runs of about equal cost (element
+ * bytes plus a fixed per-unit cost).  "Warp" below stands for whoever streams a
+ * run.  The large-unit loop shape uses exactly this cut, with max_warps = about
+ * 16 runs per warp (gnmr_info.num_runs).  The small-unit loop shape cuts into
+ * one run per resident CTA (gnmr_info.num_ctas), whose warps share it in blocks
+ * of segments that this call does not list, and departs from equal runs in two
+ * cases: arenas of at most 48 KiB of cost per resident CTA are cut between
+ * units wherever these are at most 128 KiB, and a CTA is cut shorter where its
+ * run would hold more than 2,048 blocks.  Outputs, caller-allocated: run_unit /
+ * run_pos [max_warps + 1] (run w covers (run_unit[w], run_pos[w]) up to, not
+ * including, (run_unit[w+1], run_pos[w+1])), first_warp / num_parts [num_units]
+ * (the warps touching unit b are first_warp[b] .. first_warp[b] + num_parts[b]
+ * - 1).  *num_warps receives the number of runs.  No CUDA call is made.  Errors:
  * GNMR_ERR_INVALID_ARG. */
 gnmr_status gnmr_plan_partition(int32_t num_units, const int64_t *lengths, int32_t dtype,
                                 int32_t max_warps, int32_t *num_warps, int32_t *run_unit,

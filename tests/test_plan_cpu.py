@@ -216,3 +216,18 @@ def test_plan_refuses_what_it_cannot_number(lib):
     off, unit = np.zeros(1, np.int64), np.zeros(1, np.int32)
     assert lib.plan_query(ctypes.c_int64(1), _pointer(off), _pointer(lens), _pointer(unit), ctypes.c_int32(1),
                           ctypes.c_int(2), ctypes.c_int32(CTAS), _pointer(sizes)) == 0
+
+
+@pytest.mark.parametrize("units,top,eb", [(3000, 60_000, 2), (100_000, 3000, 4), (600, 200_000, 2)])
+def test_the_public_query_gives_the_ctas_of_larger_arenas(lib, units, top, eb):
+    """gnmr_plan_partition, asked for as many runs as there are resident CTAs,
+    lists the CTAs' parts of arenas above 48 KiB of cost per CTA."""
+    from paper_2606_00539_gb300 import _native as N
+    lens = np.random.default_rng(units).integers(0, top, units).astype(np.int64)
+    assert (lens * eb + 4096).sum() > CTAS * (48 << 10)
+    p = Plan(lib, _packed(lens), lens, None, eb)
+    run_unit, _, first, parts = N.gnmr_plan_partition(lens, N.GNMR_DTYPE_BF16 if eb == 2 else N.GNMR_DTYPE_F32, CTAS)
+    assert np.array_equal(run_unit[:-1], p.cta[:, 2])
+    for ends, col in ((p.cta[:, 2], 6), (p.cta[:, 2] + p.cta[:, 3] - 1, 7)):
+        assert np.array_equal(parts[ends], p.cta[:, col])
+        assert np.array_equal(np.arange(len(ends)) - first[ends], p.cta[:, col + 2])
