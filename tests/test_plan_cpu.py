@@ -231,3 +231,18 @@ def test_the_public_query_gives_the_ctas_of_larger_arenas(lib, units, top, eb):
     for ends, col in ((p.cta[:, 2], 6), (p.cta[:, 2] + p.cta[:, 3] - 1, 7)):
         assert np.array_equal(parts[ends], p.cta[:, col])
         assert np.array_equal(np.arange(len(ends)) - first[ends], p.cta[:, col + 2])
+
+
+@pytest.mark.parametrize("units,eb,seed", [(300, 2, 1), (300, 4, 2), (500, 2, 3), (40, 4, 4)])
+def test_small_arenas_give_no_cta_two_rounds(lib, units, eb, seed):
+    """Arenas cut between units: no CTA gets more than 128 KiB, units of that and
+    more get CTAs of their own, and there is one wave of CTAs."""
+    lens = np.minimum(np.exp(np.random.default_rng(seed).normal(8, 1.8, units)).astype(np.int64), 100_000)
+    cost = lens * eb + 4096
+    assert cost.sum() <= CTAS * (48 << 10)
+    p = Plan(lib, _packed(lens), lens, None, eb)
+    check(p)
+    assert len(p.cta) <= CTAS
+    for c in p.cta:
+        b = p.block[c[4] * p.entries:(c[4] + c[5]) * p.entries]
+        assert b[b[:, 1] > 0, 1].sum() * eb + 4096 * (c[3] - (c[8] > 0)) <= (128 << 10) + 512
