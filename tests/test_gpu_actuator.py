@@ -299,7 +299,8 @@ def test_units_of_few_rows(dtype, most_rows, shift, cuda_device):
     g = torch.Generator(cuda_device).manual_seed(most_rows)
     x = torch.randn(total, device=cuda_device, generator=g).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
     x[off[14]:off[14] + rows[14] * cols[14]] = 0
-    out = torch.zeros(total + 16, dtype=x.dtype, device=cuda_device)[shift:shift + total]
+    whole = torch.full((total + 16,), 3.0, dtype=x.dtype, device=cuda_device)
+    out = whole[shift:shift + total]
     mask = (np.arange(len(rows)) % 3 == 0).astype(np.uint8)
     d_mask = torch.from_numpy(mask).to(cuda_device)
     h = N.gnmr_actuator_create(off, rows, cols, N.GNMR_DTYPE_BF16 if dtype == "bf16" else N.GNMR_DTYPE_F32, 0)
@@ -313,5 +314,10 @@ def test_units_of_few_rows(dtype, most_rows, shift, cuda_device):
         for b in range(len(rows)):
             part = slice(off[b], off[b] + rows[b] * cols[b])
             assert np.array_equal(got[part].view(word), want[part].view(word)), (b, rows[b], cols[b])
+        # nothing else is written: not between the units, nor before and behind the buffer
+        covered = np.zeros(total + 16, bool)
+        for b in range(len(rows)):
+            covered[shift + off[b]:shift + off[b] + rows[b] * cols[b]] = True
+        assert (whole.float().cpu().numpy()[~covered] == 3.0).all()
     finally:
         N.gnmr_actuator_destroy(h)

@@ -116,8 +116,8 @@ def test_loop_shape_follows_the_mean_unit_size(cuda_device):
 
 
 def test_large_unit_loop_takes_runs_dynamically(cuda_device):
-    """The large-unit loop plans about 16 runs per warp (64-256 KiB each), and
-    the small-unit loop one run per warp."""
+    """The large-unit loop plans about 16 runs per warp (64-256 KiB each); the
+    small-unit loop reports the warps that start on a block as its runs."""
     for config in ("llama2-1.3b", "llama2-13b", "moe", "tiny", "aq-stress"):
         w = workloads.make(config)
         with _monitor(w) as mon:
@@ -910,3 +910,33 @@ def test_short_units_share_a_warp(dtype, start, cuda_device):
         torch.testing.assert_close(stats["norm"], want, rtol=1e-6, atol=0, equal_nan=True)
         sums = mon.step_partials(arena)
         assert torch.equal(sums.sqrt().nan_to_num(7.0), stats["norm"].nan_to_num(7.0))
+
+
+@pytest.mark.parametrize("shape", ["small", "large", "grouped"])
+def test_lanes_are_joined_without_rounding(shape, cuda_device):
+    """One element in each lane's first vector, squares of 24 bits in [1, 2) and
+    [1/4, 1/2): the lanes' totals and their sum fit the 26-bit fractions exactly,
+    where fp32 additions over the lanes would round (1e-8)."""
+    import torch
+    rng = np.random.default_rng(3)
+    if shape == "grouped":                                # 4, 8 and 16 lanes to a unit
+        lengths = np.tile([16, 136, 264], 7000)
+        lanes = np.tile([4, 8, 16], 7000)
+    else:
+        lengths = np.full(64, 128)
+        lanes = np.full(64, 32)
+    offsets = np.cumsum(lengths) - lengths                # multiples of 8 elements: no head
+    lane = np.arange(lanes.sum()) - np.repeat(np.cumsum(lanes) - lanes, lanes)
+    x = (1 + rng.integers(1, 800, len(lane)) * 2.0 ** -11) * rng.choice([1.0, 0.5], len(lane))
+    host = np.zeros(int(lengths.sum()), np.float32)
+    host[np.repeat(offsets, lanes) + 4 * lane] = x        # exact in 12 bits
+    want = np.sqrt(np.add.reduceat(x * x, np.cumsum(lanes) - lanes))      # exact sums, one rounding
+    with Monitor(offsets, lengths, dtype="f32", window=2, loop_shape="large" if shape == "large" else "small") as mon:
+        stats = mon.new_stats()
+        arena = torch.from_numpy(host).to(cuda_device)
+        mon.step(arena, stats=stats)
+        # a unit that two CTAs share is cut where fewer lanes may hold more of it
+        cut = mon.info()["num_ctas"] - 1 if shape == "grouped" else 0
+        for got in (stats["norm"].cpu().numpy(), np.sqrt(mon.step_partials(arena).cpu().numpy())):
+            assert (got != want).sum() <= cut
+            np.testing.assert_allclose(got, want, rtol=2.0 ** -22, atol=0)
