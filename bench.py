@@ -217,8 +217,8 @@ def grid_text(info) -> str:
     if info["loop_shape"] == 2:
         return (f"{info['num_ctas']} CTAs x {info['threads_per_cta']} threads, {info['num_runs']} runs "
                 f"taken dynamically by {info['num_warps']} warps, large-unit loop shape")
-    return (f"{info['num_ctas']} CTAs x {info['threads_per_cta']} threads, {info['num_warps']} warp runs, "
-            f"small-unit loop shape")
+    return (f"{info['num_ctas']} CTAs x {info['threads_per_cta']} threads, {info['num_warps']} warps "
+            f"start on a block, small-unit loop shape")
 
 
 def measured_peaks():

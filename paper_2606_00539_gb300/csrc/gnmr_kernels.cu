@@ -4,13 +4,14 @@
 // more segments of the arena) is cut by gnmr_plan.cpp.  For every piece of a
 // segment the warp streams the gradient with 16-byte loads (8 or 16 in flight
 // per lane, by the loop shape), squares in fp32, sums blocks of 16 iterations
-// in fp32 and the blocks as float pairs (error-free TwoSum), and all-reduces
-// the lanes' totals across the warp with shuffles, converting to fp64 once per
-// piece: n_b = ||g_b||_2 (Sec. 2, Eq. local_gradient).  (The streaming
-// reduction lives in gnmr_stream.cuh.)
+// in fp32 and the blocks as float pairs (error-free TwoSum), and adds the
+// lanes' totals across the warp in fixed point, by integer reductions, forming
+// the fp64 result once per piece: n_b = ||g_b||_2 (Sec. 2, Eq. local_gradient).
+// (The streaming reduction lives in gnmr_stream.cuh.)
 //
 // Small-unit loop: a CTA owns a contiguous part of the stream, cut into blocks
-// of 8 KiB and less, which its warps take from a counter in shared memory.
+// (8 KiB at most; about 16 KiB in layouts of units of 128 KiB and more, and more
+// where a CTA has too many), which its warps take from a counter in shared memory.
 // HBM serves warps unevenly (with one fixed run per warp the first warps of a
 // 125 MB step ended after 13 us and the last after 29), so warps that stream
 // faster take more blocks; a block's sum goes to a slot in shared memory, and
@@ -69,11 +70,12 @@
 namespace gnmr {
 namespace {
 
-// Two compiled shapes of the streaming loop, chosen per handle from the mean
-// unit size (both measured on GB300): small units run best with 8
-// 16-byte loads in flight per lane and two CTAs per SM; large units with 16
-// loads per lane and one CTA per SM (fewer, deeper streams) and runs of at
-// most 256 KiB taken dynamically.
+// Three compiled shapes of the streaming loop, chosen per handle from the unit
+// and arena sizes (measured on GB300): small units and arenas run best with 8
+// 16-byte loads in flight per lane and two CTAs per SM, with a variant for
+// layouts where short blocks dominate, several of them to a warp; large units
+// with 16 loads per lane and one CTA per SM (fewer, deeper streams) and runs of
+// at most 256 KiB taken dynamically.
 template <int V> struct Shape;
 template <> struct Shape<kVariantSmall> {
     static constexpr int kUnroll = 8;

@@ -14,8 +14,9 @@
 //
 // The array (kScratchBytes, about 5.6 MiB) is reserved on every GPU that
 // loads the library until the process exits.  Every call shares it and it
-// keeps the last call's contents; the per-unit tickets that must start at
-// zero are cleared by each call.  Calls whose work overlaps on the GPU (two
+// keeps the last call's contents; the per-unit tickets, which must start at
+// zero, are cleared by each call that uses them (layouts in which several warps
+// share a unit).  Calls whose work overlaps on the GPU (two
 // streams, or two host threads) race on the array: serialise them.
 #include <cmath>
 #include <cstdint>
