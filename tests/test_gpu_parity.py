@@ -940,3 +940,27 @@ def test_lanes_are_joined_without_rounding(shape, cuda_device):
         for got in (stats["norm"].cpu().numpy(), np.sqrt(mon.step_partials(arena).cpu().numpy())):
             assert (got != want).sum() <= cut
             np.testing.assert_allclose(got, want, rtol=2.0 ** -22, atol=0)
+
+
+@pytest.mark.parametrize("shape", ["small", "large"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("start", [0, 1])
+def test_ends_of_pieces(dtype, shape, start, cuda_device):
+    """Units that end around every length of the last round of loads: whole
+    numbers, whose sums of squares no rounding touches, come out exact."""
+    import torch
+    per = 4 if dtype == "f32" else 8
+    vecs = [v + d for v in (0, 32, 64, 96, 128, 160, 192, 224, 256, 384, 448, 512, 768, 1024) for d in (-1, 0, 1) if v + d >= 0]
+    lengths = np.array([v * per + e for v in vecs for e in (0, 1, per - 1)], np.int64)
+    offsets = start + np.cumsum(lengths) - lengths
+    n = int(offsets[-1] + lengths[-1])
+    g = torch.Generator(cuda_device).manual_seed(11)
+    x = torch.randint(-3, 4, (n,), device=cuda_device, generator=g)
+    ids = torch.repeat_interleave(torch.arange(len(lengths), device=cuda_device), torch.from_numpy(lengths).to(cuda_device))
+    want = torch.zeros(len(lengths), dtype=torch.float64, device=cuda_device).index_add_(0, ids, x[start:].double().square())
+    arena = x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    with Monitor(offsets, lengths, dtype=dtype, window=2, loop_shape=shape) as mon:
+        stats = mon.new_stats()
+        mon.step(arena, stats=stats)
+        assert torch.equal(stats["norm"], want.sqrt())
+        assert torch.equal(mon.step_partials(arena), want)
