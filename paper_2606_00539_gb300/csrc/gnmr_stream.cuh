@@ -16,7 +16,7 @@
 // layout (normal values): fp32 units of 8 KB 3.7e-9, of 120 KB 9.5e-10, of 1.2 MB
 // 4.3e-10, of 12 MB 3.3e-10; with an fp32 tree over the lanes (and one run per warp
 // in the small-unit loop) 1.9e-8, 1.2e-8, 3.7e-9 and 1.5e-9.  bf16 units: 5.7e-9 to
-// 6.8e-9 at every size, with the tree 6.1e-9 (units of 6 MB) to 2.0e-8 (4 KB).  What
+// 6.6e-9 at every size, with the tree 6.1e-9 (units of 6 MB) to 2.0e-8 (4 KB).  What
 // is left there is a common offset of about -5.8e-9, the same as with the tree,
 // whose scatter lay around it: a bf16 square ends in the bits 001 or in zeros, so
 // rounding the first sums of a few to fp32 drops more than it adds.
